@@ -50,6 +50,7 @@ thread_local std::string g_create_err;
 // refinement steps before the float64 kernel takes over.
 constexpr double kMixedInnerTol = 1e-5;
 constexpr int kMaxRefine = 8;
+const char* const kBarrierTimeout = "grid-wide PCG barrier timed out";
 
 enum {
   DS_UN2 = 0, DS_VN2 = 1, DS_NB = 2, DS_NA = 3, DS_DW = 4, /*5*/ DS_ZKZ = 6, DS_ZF = 7, DS_RN = 8, DS_V0 = 9,
@@ -180,6 +181,7 @@ struct cr_problem {
   std::vector<std::pair<void*, size_t>> allocs;
   DevLap Lx, Ly;
   DevMg mg[2];  // multigrid hierarchies of L_y (side 0) and L_x (side 1)
+  DevMgGrid mgg[2];  // their grid-wide form (nb = 0: the cluster kernel)
   int *xc_ptr = nullptr, *xc_row = nullptr;
   double* xc_val = nullptr;
   DevXLocal xl;
@@ -554,6 +556,129 @@ cr_status build_lap(cr_problem* p, const cr_csr& c, DevLap& L) {
   return CR_OK;
 }
 
+// Grid-wide form of the multigrid PCG (cr_mg_grid.cu) on the hierarchy H.  It
+// takes every SM in a cooperative launch, so it serves the problems that have
+// the GPU to themselves: one that caps its persistent Galerkin kernel
+// (galerkin_ctas, as the members of a sweep do) or asks for a cluster size
+// keeps the cluster kernel, of which many run side by side.  Leaves d.nb = 0
+// where it does not apply.
+cr_status build_mg_grid(cr_problem* p, const DevLap& L, const cr_mg::Hierarchy& H, const DevMg& h, DevMgGrid& out) {
+  out = DevMgGrid{};
+  if (p->opt.galerkin_ctas > 0 || p->opt.cluster_size > 0) return CR_OK;
+  int dev = 0, sms = 0, coop = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  if (!coop || sms < 1) return CR_OK;
+  const int n = h.lev[0].n, nlev = h.nlev, nc = h.nc, m = p->m;
+  DevMgGrid d{};
+  d.nb = std::min(sms, std::max(1, (n + kMgGridRows - 1) / kMgGridRows));
+  for (int l = 0; l < nlev; ++l) d.lev[l].chunk = (h.lev[l].n + d.nb - 1) / d.nb;
+  d.threads = kMgGridThreads;
+  // lanes per row: eight entries of a row are in flight per lane, so that most rows take one trip to L2
+  auto lanes = [&](const std::vector<int>& rp, int rows, int threads) {
+    int64_t mx = 0;
+    for (size_t r = 0; r + 1 < rp.size(); ++r) mx = std::max<int64_t>(mx, rp[r + 1] - rp[r]);
+    int g = 1;
+    while (g < 32 && 8 * g < mx && 2 * g * rows <= threads) g *= 2;
+    return g;
+  };
+  // entries of the busiest CTA: rows [b chunk, (b + 1) chunk) of a CSR
+  auto most = [&](const std::vector<int>& rp, int chunk) {
+    const int rows = (int)rp.size() - 1;
+    int mx = 0;
+    for (int r = 0; r < rows; r += chunk) mx = std::max(mx, rp[std::min(rows, r + chunk)] - rp[r]);
+    return mx;
+  };
+  int64_t sm = 0;
+  auto sect = [&](int64_t bytes) {
+    const int64_t at = sm;
+    sm += (bytes + 15) / 16 * 16;
+    return (int)at;
+  };
+  d.o_m = sect(8 * (2 * (int64_t)m + (h.smw ? (int64_t)m * m + m : 0)));
+  for (int l = 0; l < nlev - 1; ++l)
+    d.lev[l].o_own = sect(8 * (int64_t)(l == 0 ? kMgGridOwn0 : kMgGridOwn) * d.lev[l].chunk);
+  d.o_tab = (int)sm;
+  sm = 0;
+  d.o_nb = sect(4 * (int64_t)L.K * d.lev[0].chunk);
+  d.o_nbw = L.offw ? sect(8 * (int64_t)L.K * d.lev[0].chunk) : -1;
+  for (int l = 0; l < nlev - 1; ++l) {
+    const cr_mg::Level& HL = H.lev[l];
+    DevMgGridLevel& W = d.lev[l];
+    if (l >= 1) {
+      const cr_mg::Triple u = cr_mg::unite(HL.L, HL.M, HL.M);  // the operator rows as uploaded
+      const int e = most(u.rp, W.chunk);
+      W.g_op = lanes(u.rp, W.chunk, d.threads / 2);
+      W.o_rp = sect(4 * (int64_t)(W.chunk + 1));
+      W.o_ci = sect(4 * (int64_t)e);
+      W.o_cv = sect(8 * (int64_t)e);
+    }
+    const cr_mg::Triple S = cr_mg::unite(HL.P, HL.LP, HL.MP), T = cr_mg::transpose(S);
+    W.g_t = lanes(T.rp, d.lev[l + 1].chunk, d.threads / 2);
+    W.g_s = l < nlev - 2 ? lanes(S.rp, W.chunk, d.threads) : lanes({0, nc}, W.chunk, d.threads);
+    if (l < nlev - 2) {
+      const int e = most(S.rp, W.chunk);
+      W.o_srp = sect(4 * (int64_t)(W.chunk + 1));
+      W.o_sci = sect(4 * (int64_t)e);
+      W.o_scv = sect(8 * (int64_t)e);
+    } else {
+      W.o_scv = sect(8 * (int64_t)W.chunk * nc);
+      W.o_sq = sect(8 * (int64_t)W.chunk * nc);
+    }
+    const int chunk1 = d.lev[l + 1].chunk, e = most(T.rp, chunk1);
+    W.o_trp = sect(4 * (int64_t)(chunk1 + 1));
+    W.o_tci = sect(4 * (int64_t)e);
+    W.o_tcv = sect(8 * (int64_t)e);
+    int *d1 = nullptr, *d2 = nullptr, *d3 = nullptr, *d4 = nullptr;
+    double *v1 = nullptr, *v2 = nullptr, *v3 = nullptr, *v4 = nullptr, *v5 = nullptr, *v6 = nullptr;
+    TRY(upload(p, &d1, S.rp));
+    TRY(upload(p, &d2, S.ci));
+    TRY(upload(p, &v1, S.a));
+    TRY(upload(p, &v2, S.b));
+    TRY(upload(p, &v3, S.c));
+    TRY(upload(p, &d3, T.rp));
+    TRY(upload(p, &d4, T.ci));
+    TRY(upload(p, &v4, T.a));
+    TRY(upload(p, &v5, T.b));
+    TRY(upload(p, &v6, T.c));
+    CUCHK(p, cudaStreamSynchronize(p->st));  // S and T leave scope
+    W.srp = d1;
+    W.sci = d2;
+    W.sp = v1;
+    W.sl = v2;
+    W.sm = v3;
+    W.trp = d3;
+    W.tci = d4;
+    W.tp = v4;
+    W.tl = v5;
+    W.tm = v6;
+    double* g = nullptr;
+    TRY(dalloc(p, &g, (size_t)6 * h.lev[l].n));
+    W.g = g;
+    TRY(dalloc(p, &W.dinv, (size_t)h.lev[l].n));
+  }
+  d.tab_bytes = (int)sm;
+  d.tab_smem = (int64_t)d.o_tab + sm <= kMgGridSmemMax ? 1 : 0;
+  d.smem = (size_t)d.o_tab + (d.tab_smem ? (size_t)sm : 0);
+  if (d.smem > (size_t)kMgGridSmemMax) return CR_OK;
+  if (!mg_grid_prepare(d)) return CR_OK;
+  if (!d.tab_smem) TRY(dalloc(p, &d.tab_glob, (size_t)d.nb * d.tab_bytes));
+  double* rc = nullptr;
+  TRY(dalloc(p, &rc, (size_t)nc));
+  d.rc = rc;
+  TRY(dalloc(p, &d.ytot, (size_t)m));
+  TRY(dalloc(p, &d.part, (size_t)4 * d.nb));
+  if (h.smw) {
+    TRY(dalloc(p, &d.smw_lmx, (size_t)n * m));
+    TRY(dalloc(p, &d.smw_rows, (size_t)3 * n * m));
+  }
+  TRY(dalloc(p, &d.bar, 2));
+  d.err = reinterpret_cast<int*>(d.bar + 1);
+  out = d;
+  return CR_OK;
+}
+
 // Multigrid hierarchy of one Laplacian (cr_mg_host.h) on the cluster partition
 // of L: level 0 in L's chunks, larger coarse levels in equal chunks over the
 // cluster, levels of at most kMgTailRows rows and the coarsest (at most
@@ -759,6 +884,8 @@ cr_status build_mg(cr_problem* p, const cr_csr& c, const DevLap& L, DevMg& g) {
   }
   h.tab_bytes = tb;
   h.smw = (&g == &p->mg[1] && p->m <= kMgSmwMax) ? 1 : 0;  // v side, small enough data term
+  DevMgGrid& gg = p->mgg[&g == &p->mg[1] ? 1 : 0];
+  TRY(build_mg_grid(p, L, H, h, gg));
   const size_t cap = 227 * 1024;
   bool need_glob = false;
   for (int f = 0; f < 2; ++f) {
@@ -768,13 +895,17 @@ cr_status build_mg(cr_problem* p, const cr_csr& c, const DevLap& L, DevMg& g) {
     h.smem[f] = with <= cap ? with : (without <= cap ? without : 0);
     if (h.smem[f] && !h.tab_smem[f]) need_glob = true;
   }
-  if (need_glob) TRY(dalloc(p, &h.tab_glob, (size_t)C * h.tab_bytes));
+  if (need_glob && gg.nb == 0) TRY(dalloc(p, &h.tab_glob, (size_t)C * h.tab_bytes));
   if (h.smw) {
     // the cache of the v side's Sherman-Morrison-Woodbury correction; smw_sig = {shift, precision}
     // of the MX it holds (0: none), so a launch of either precision knows whether to rebuild it
     TRY(dalloc(p, &h.smw_mx, (size_t)n * p->m));
     TRY(dalloc(p, &h.smw_xx, (size_t)p->m * p->m));
     TRY(dalloc(p, &h.smw_sig, 3));
+  }
+  if (gg.nb > 0) {
+    g = h;
+    return CR_OK;
   }
   if (h.smem[0] == 0 && h.smem[1] == 0) return CR_OK;
   CUCHK(p, mg_prepare());
@@ -998,7 +1129,7 @@ constexpr double kMgAutoLambda = 1e3;
 
 bool use_mg(const cr_problem* p, int side, bool fp32) {
   const DevMg& g = p->mg[side];
-  if (!(g.nlev >= 2 && g.smem[fp32 ? 0 : 1] > 0)) return false;
+  if (!(g.nlev >= 2 && (p->mgg[side].nb > 0 || g.smem[fp32 ? 0 : 1] > 0))) return false;
   if (p->opt.precond == CR_PRECOND_MULTIGRID) return true;
   if (p->opt.precond != CR_PRECOND_AUTO) return false;
   // measured on GB300 (7,530 voxels): a multigrid iteration costs ~80-125 us (float32) / ~90-165 us
@@ -1012,7 +1143,15 @@ cr_status run_pcg(cr_problem* p, int side, const double* b, double* x, int maxit
   const int kph = side == 0 ? CR_PHASE_PCG_KERNEL : CR_PHASE_PCG_KERNEL_V;
   if (use_mg(p, side, fp32)) {
     prof_begin(p, kph);
-    CUCHK(p, mg_pcg_launch(pcg_args(p, side, b, x, maxit, tol, fp32), p->mg[side], side, p->st));
+    if (p->mgg[side].nb > 0) {
+      DevMgGrid d = p->mgg[side];
+      d.xc_ptr = p->xc_ptr;
+      d.xc_row = p->xc_row;
+      d.xc_val = p->xc_val;
+      CUCHK(p, mg_grid_launch(pcg_args(p, side, b, x, maxit, tol, fp32), p->mg[side], d, side, p->st));
+    } else {
+      CUCHK(p, mg_pcg_launch(pcg_args(p, side, b, x, maxit, tol, fp32), p->mg[side], side, p->st));
+    }
     prof_end(p, kph);
     return CR_OK;
   }
@@ -1046,7 +1185,7 @@ cr_status run_pcg(cr_problem* p, int side, const double* b, double* x, int maxit
                            p->pg_yglob, p->pg_bar, p->pg_err, std::min(nb, std::max(1, L.n / 64)), p->st));
   prof_end(p, kph);
   TRY(readback(p, 0, 1, true));
-  if (p->hs->stat[side].status == 3) return fail(p, CR_ETIMEOUT, "grid-wide PCG barrier timed out");
+  if (p->hs->stat[side].status == 3) return fail(p, CR_ETIMEOUT, kBarrierTimeout);
   return CR_OK;
 }
 
@@ -1098,6 +1237,7 @@ cr_status launch_pcg_mixed(cr_problem* p, int side, const double* b, double* x, 
       TRY(run_pcg(p, side, b, x, std::max(1, maxit - total), tol, false));
       TRY(readback(p, 0, 1, true));
       hs = p->hs->stat[side];
+      if (hs.status == 3) return fail(p, CR_ETIMEOUT, kBarrierTimeout);
       hs.iters += total;
       break;
     }
@@ -1109,6 +1249,7 @@ cr_status launch_pcg_mixed(cr_problem* p, int side, const double* b, double* x, 
     TRY(run_pcg(p, side, r, d, maxit - total, inner, true));
     TRY(readback(p, 0, 1, true));
     const PcgStat in = p->hs->stat[side];
+    if (in.status == 3) return fail(p, CR_ETIMEOUT, kBarrierTimeout);
     total += in.iters;
     hs.iters = total;
     if (in.status == 2) {
@@ -1763,6 +1904,7 @@ cr_status do_rank_one(cr_problem* p, cr_rank1_info* info) {
     scale_by_inv_norm(nx, p->vhat, p->ds + DS_VN2, p->v, st);
     TRY(readback(p, 0, 2, true));
     const PcgStat* s = p->hs->stat;
+    if (s[0].status == 3 || s[1].status == 3) return fail(p, CR_ETIMEOUT, kBarrierTimeout);
     p->pcg_solves += 2;
     p->pcg_iters += s[0].iters + s[1].iters;
     p->pcg_iters_side[0] += s[0].iters;
@@ -2324,7 +2466,8 @@ cr_status cr_get_stats(cr_problem* p, cr_stats* s, int32_t reset) {
   for (int side = 0; side < 2; ++side) {
     const DevLap& L = side == 0 ? p->Ly : p->Lx;
     const bool f32 = p->opt.precision == CR_MIXED;
-    s->pcg_cluster[side] = (use_mg(p, side, f32) || !use_grid_pcg(p, side, f32)) ? L.csize : 0;
+    const bool mg = use_mg(p, side, f32);
+    s->pcg_cluster[side] = (mg ? p->mgg[side].nb == 0 : !use_grid_pcg(p, side, f32)) ? L.csize : 0;
     s->pcg_multigrid[side] = use_mg(p, side, f32) ? p->mg[side].nlev : 0;
   }
   s->galerkin_eigen[0] = p->gal_eig_proj;
@@ -2781,6 +2924,7 @@ cr_status cr_solve_u(cr_problem* p, const double* v, const double* rhs, double* 
   CUCHK(p, cudaMemcpyAsync(uh, p->uhat, sizeof(double) * p->ny, cudaMemcpyDeviceToHost, st));
   TRY(readback(p, 0, 1, true));
   if (iters) *iters = p->hs->stat[0].iters;
+  if (p->hs->stat[0].status == 3) return fail(p, CR_ETIMEOUT, kBarrierTimeout);
   if (p->hs->stat[0].status == 2) return fail(p, CR_ENOTCONV, "PCG breakdown");
   if (p->hs->stat[0].status == 1) return fail(p, CR_ENOTCONV, "PCG reached pcg_maxit");
   return CR_OK;
@@ -2797,6 +2941,7 @@ cr_status cr_solve_v(cr_problem* p, const double* u, const double* rhs, double* 
   CUCHK(p, cudaMemcpyAsync(vh, p->vhat, sizeof(double) * p->nx, cudaMemcpyDeviceToHost, st));
   TRY(readback(p, 0, 1, true));
   if (iters) *iters = p->hs->stat[1].iters;
+  if (p->hs->stat[1].status == 3) return fail(p, CR_ETIMEOUT, kBarrierTimeout);
   if (p->hs->stat[1].status == 2) return fail(p, CR_ENOTCONV, "PCG breakdown");
   if (p->hs->stat[1].status == 1) return fail(p, CR_ENOTCONV, "PCG reached pcg_maxit");
   return CR_OK;

@@ -203,6 +203,48 @@ bool mg_cluster_ok(int csize, size_t smem, bool fp32);
 // partition of a.L.  a.x is the initial guess and the result; a.p, a.sv, a.omt are work.
 cudaError_t mg_pcg_launch(const PcgArgs& a, const DevMg& g, int side, cudaStream_t st);
 
+// ---------------------------------------------------------------- cr_mg_grid.cu
+// The same preconditioned PCG over all SMs (one cooperative launch): per level
+// the row split, the smoothed transfer S_l = P - w D^-1 (L + sigma M) P (rows
+// of level l, columns of level l+1) by its three parts on one pattern, its
+// transpose, and where the level's vectors and tables lie.
+constexpr int kMgGridThreads = 512;
+constexpr int kMgGridRows = 16;               // fewest level-0 rows per CTA
+constexpr int kMgGridSmemMax = 224 * 1024;    // dynamic shared memory (about 1 KB is static)
+constexpr int kMgGridOwn0 = 16, kMgGridOwn = 7;  // own vectors of level 0 and of the levels below
+struct DevMgGridLevel {
+  int chunk = 0;  // rows per CTA
+  const int *srp = nullptr, *sci = nullptr;  // S_l by rows
+  const double *sp = nullptr, *sl = nullptr, *sm = nullptr;
+  const int *trp = nullptr, *tci = nullptr;  // S_l^T by rows of level l+1
+  const double *tp = nullptr, *tl = nullptr, *tm = nullptr;
+  double* dinv = nullptr;  // 1 / diag(L + sigma M)
+  void* g = nullptr;       // published vectors (n entries each)
+  int o_own = 0;           // bytes from the start of shared memory
+  int g_op = 1, g_s = 1, g_t = 1;  // lanes per row of the operator, S and S^T tables
+  // bytes from the table base: operator rows, S rows (the dense S (L_c + sigma M_c)^-1 on the
+  // level above the coarsest, with its workspace o_sq), S^T rows (rows of level l+1)
+  int o_rp = 0, o_ci = 0, o_cv = 0, o_srp = 0, o_sci = 0, o_scv = 0, o_sq = 0, o_trp = 0, o_tci = 0, o_tcv = 0;
+};
+struct DevMgGrid {
+  int nb = 0, threads = 0;  // CTAs (0: not available) and threads per CTA
+  DevMgGridLevel lev[kMgMaxLev];
+  int o_m = 0, o_nb = 0, o_nbw = -1, o_tab = 0;
+  int tab_smem = 0, tab_bytes = 0;
+  size_t smem = 0;
+  char* tab_glob = nullptr;
+  void* rc = nullptr;         // coarsest right side
+  double *ytot = nullptr, *part = nullptr;
+  double* smw_lmx = nullptr;   // v side, smw: L MX, beside DevMg::smw_mx
+  double* smw_rows = nullptr;  // v side, smw: per row [MX Q | (L + cI) MX Q | X Q] (3 m values of the working precision)
+  unsigned* bar = nullptr;  // the barrier's counter, then its error word
+  int* err = nullptr;
+  const int *xc_ptr = nullptr, *xc_row = nullptr;  // v side: X by columns (set at the launch)
+  const double* xc_val = nullptr;
+};
+bool mg_grid_prepare(const DevMgGrid& d);
+cudaError_t mg_grid_launch(const PcgArgs& a, const DevMg& g, const DevMgGrid& d, int side, cudaStream_t st);
+
 // ---------------------------------------------------------------- cr_pcg_grid.cu
 // Grid-wide PCG (vectors in HBM, all SMs) for grids the register-resident cluster kernel does not take.
 // Blocks of the cooperative launch (0: cannot run) and work doubles needed.

@@ -200,7 +200,65 @@ inline Csr prolongation(const Csr& A, const std::vector<int>& agg, int n_agg, do
 struct Level {
   Csr L, M;  // level operators: the kernel smooths with L + sigma M
   Csr P, R;  // prolongation from the next level (rows x next rows) and R = P^T (empty on the last level)
+  Csr LP, MP;  // L P and M P (empty on the last level)
 };
+
+// Three matrices on the union of their patterns: columns ascending, a value of each per entry.
+struct Triple {
+  int rows = 0, cols = 0;
+  std::vector<int> rp{0}, ci;
+  std::vector<double> a, b, c;
+};
+
+inline Triple unite(const Csr& A, const Csr& B, const Csr& C) {
+  Triple t;
+  t.rows = A.rows;
+  t.cols = A.cols;
+  t.rp.assign(A.rows + 1, 0);
+  const size_t cap = std::max(A.ci.size(), std::max(B.ci.size(), C.ci.size())) + A.ci.size() / 4;
+  t.ci.reserve(cap);
+  t.a.reserve(cap);
+  t.b.reserve(cap);
+  t.c.reserve(cap);
+  for (int i = 0; i < A.rows; ++i) {
+    int p = A.rp[i], q = B.rp[i], r = C.rp[i];
+    for (;;) {
+      const int ca = p < A.rp[i + 1] ? A.ci[p] : INT32_MAX, cb = q < B.rp[i + 1] ? B.ci[q] : INT32_MAX,
+                cc = r < C.rp[i + 1] ? C.ci[r] : INT32_MAX;
+      const int col = std::min(ca, std::min(cb, cc));
+      if (col == INT32_MAX) break;
+      t.ci.push_back(col);
+      t.a.push_back(ca == col ? A.v[p++] : 0.0);
+      t.b.push_back(cb == col ? B.v[q++] : 0.0);
+      t.c.push_back(cc == col ? C.v[r++] : 0.0);
+    }
+    t.rp[i + 1] = (int)t.ci.size();
+  }
+  return t;
+}
+
+inline Triple transpose(const Triple& A) {
+  Triple t;
+  t.rows = A.cols;
+  t.cols = A.rows;
+  t.rp.assign(A.cols + 1, 0);
+  for (int c : A.ci) t.rp[c + 1] += 1;
+  for (int c = 0; c < A.cols; ++c) t.rp[c + 1] += t.rp[c];
+  t.ci.resize(A.ci.size());
+  t.a.resize(A.ci.size());
+  t.b.resize(A.ci.size());
+  t.c.resize(A.ci.size());
+  std::vector<int> pos(t.rp.begin(), t.rp.end() - 1);
+  for (int i = 0; i < A.rows; ++i)
+    for (int q = A.rp[i]; q < A.rp[i + 1]; ++q) {
+      const int p = pos[A.ci[q]]++;
+      t.ci[p] = i;
+      t.a[p] = A.a[q];
+      t.b[p] = A.b[q];
+      t.c[p] = A.c[q];
+    }
+  return t;
+}
 
 struct Hierarchy {
   std::vector<Level> lev;  // lev.back() is the coarsest level (dense solve)
@@ -280,8 +338,10 @@ inline Hierarchy build(const Csr& L, int coarse_max = 64, int max_levels = 8, do
     f.P = prolongation(f.L, agg, na, omega);
     f.R = transpose(f.P);
     Level c;
-    c.L = multiply(f.R, multiply(f.L, f.P));
-    c.M = multiply(f.R, multiply(f.M, f.P));
+    f.LP = multiply(f.L, f.P);
+    f.MP = h.lev.size() == 1 ? f.P : multiply(f.M, f.P);  // M_0 = I
+    c.L = multiply(f.R, f.LP);
+    c.M = multiply(f.R, f.MP);
     h.lev.push_back(std::move(c));
   }
   return h;
