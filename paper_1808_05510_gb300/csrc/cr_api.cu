@@ -181,6 +181,7 @@ struct cr_problem {
   std::vector<std::pair<void*, size_t>> allocs;
   DevLap Lx, Ly;
   DevMg mg[2];  // multigrid hierarchies of L_y (side 0) and L_x (side 1)
+  DevPush push[2];  // float32 cluster PCG of the u side (L_y) and the v side (L_x)
   DevMgGrid mgg[2];  // their grid-wide form (nb = 0: the cluster kernel)
   int *xc_ptr = nullptr, *xc_row = nullptr;
   double* xc_val = nullptr;
@@ -462,6 +463,163 @@ cr_status check_csr(const cr_csr& c, int64_t n, const char* name, std::string& e
   return CR_OK;
 }
 
+// Tables of the float32 cluster PCG (cr_pcg_push.cu) for a unit-weight Laplacian
+// with rows[i] its off-diagonal entries, on the cluster partition of L.  Leaves
+// csize = 0 where the kernel does not apply.
+cr_status build_push(cr_problem* p, const std::vector<std::vector<std::pair<int, double>>>& rows,
+                     const std::vector<double>& diag, const DevLap& L, DevPush& out) {
+  out = DevPush{};
+  const int n = L.n, C = L.csize, chunk = L.chunk;
+  if (p->opt.precision != CR_MIXED || L.offw || L.K > 6 || C < 1 || chunk > 4 * kPcgThreads) return CR_OK;
+  DevPush d{};
+  d.chunk = chunk;
+  std::vector<std::vector<int>> ext(C), hop1(C);
+  std::vector<int> mark(n, -1), pos(n, 0), hcnt(C, 0);
+  int emax = 0;
+  for (int r = 0; r < C; ++r) {
+    const int b = std::min(n, r * chunk), e = std::min(n, b + chunk);
+    auto add = [&](int i, std::vector<int>& to) {
+      for (const auto& q : rows[i])
+        if ((q.first < b || q.first >= e) && mark[q.first] != r) {
+          mark[q.first] = r;
+          to.push_back(q.first);
+        }
+    };
+    for (int i = b; i < e; ++i) add(i, hop1[r]);
+    std::vector<int> hop2;
+    for (int i : hop1[r]) add(i, hop2);
+    ext[r] = hop1[r];
+    ext[r].insert(ext[r].end(), hop2.begin(), hop2.end());
+    std::sort(ext[r].begin(), ext[r].end());
+    hcnt[r] = (int)hop1[r].size();
+    d.hmax = std::max(d.hmax, hcnt[r]);
+    emax = std::max(emax, (int)ext[r].size());
+  }
+  d.ext = chunk + emax + 1;
+  if (d.ext > 65535) return CR_OK;
+  std::vector<uint4> own(n), hn((size_t)C * std::max(1, d.hmax), uint4{0, 0, 0, 0});
+  std::vector<double> hd((size_t)C * std::max(1, d.hmax), 0.0);
+  std::vector<std::vector<uint32_t>> dest(n);
+  for (int r = 0; r < C; ++r) {
+    const int b = std::min(n, r * chunk), e = std::min(n, b + chunk);
+    for (size_t k = 0; k < ext[r].size(); ++k) {
+      pos[ext[r][k]] = (int)k;
+      dest[ext[r][k]].push_back(((uint32_t)r << 16) | (uint32_t)(chunk + k));
+    }
+    auto number = [&](int i) { return (uint32_t)(i >= b && i < e ? i - b : chunk + pos[i]); };
+    auto six = [&](int i) {
+      uint32_t q[6];
+      for (int k = 0; k < 6; ++k) q[k] = k < (int)rows[i].size() ? number(rows[i][k].first) : (uint32_t)(d.ext - 1);
+      return uint4{q[0] | q[1] << 16, q[2] | q[3] << 16, q[4] | q[5] << 16, number(i)};
+    };
+    for (int i = b; i < e; ++i) own[i] = six(i);
+    for (int k = 0; k < hcnt[r]; ++k) {
+      hn[(size_t)r * d.hmax + k] = six(hop1[r][k]);
+      hd[(size_t)r * d.hmax + k] = diag[hop1[r][k]];
+    }
+  }
+  for (int i = 0; i < n; ++i) d.P = std::max(d.P, (int)dest[i].size());
+  std::vector<uint32_t> push((size_t)C * d.P * chunk, 0xFFFFFFFFu);
+  for (int i = 0; i < n; ++i)
+    for (size_t k = 0; k < dest[i].size(); ++k)
+      push[((size_t)(i / chunk) * d.P + k) * chunk + i % chunk] = dest[i][k];
+  uint4 *d1 = nullptr, *d2 = nullptr;
+  int* d3 = nullptr;
+  double* d4 = nullptr;
+  uint32_t* d5 = nullptr;
+  TRY(upload(p, &d1, own));
+  TRY(upload(p, &d2, hn));
+  TRY(upload(p, &d3, hcnt));
+  TRY(upload(p, &d4, hd));
+  TRY(upload(p, &d5, push));
+  CUCHK(p, cudaStreamSynchronize(p->st));  // the host tables leave scope
+  d.own = d1;
+  d.hn = d2;
+  d.hcnt = d3;
+  d.hdiag = d4;
+  d.push = d5;
+  d.csize = C;
+  out = d;
+  return CR_OK;
+}
+
+// The v side's part of the tables: X by columns (cp, row, val) and by rows (rp, rc, rv).
+cr_status build_push_x(cr_problem* p, DevPush& d, const std::vector<int>& cp, const std::vector<int>& row,
+                       const std::vector<double>& val, const std::vector<int>& rp, const std::vector<int>& rc,
+                       const std::vector<double>& rv) {
+  if (d.csize < 1) return CR_OK;
+  const int C = d.csize, chunk = d.chunk, n = p->nx, m = p->m;
+  std::vector<int> qoff(C + 1, 0), aoff(C + 1, 0), eoff(C + 1, 0), rq((size_t)C * (chunk + 1), 0), acol, abeg;
+  std::vector<float4> qv;
+  std::vector<ushort4> qc;
+  std::vector<uint16_t> er;
+  std::vector<float> ev;
+  std::vector<int> at(cp.begin(), cp.end() - 1);  // the next entry of each column (rows ascend)
+  d.xq_max = 0;
+  for (int r = 0; r < C; ++r) {
+    const int b = std::min(n, r * chunk), e = std::min(n, b + chunk);
+    for (int li = 0; li < chunk; ++li) {
+      rq[(size_t)r * (chunk + 1) + li] = (int)qv.size() - qoff[r];
+      if (b + li >= e) continue;
+      for (int q = rp[b + li]; q < rp[b + li + 1]; q += 4) {
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+        unsigned short c[4] = {0, 0, 0, 0};
+        for (int k = 0; k < 4 && q + k < rp[b + li + 1]; ++k) {
+          v[k] = (float)rv[q + k];
+          c[k] = (unsigned short)rc[q + k];
+        }
+        qv.push_back(float4{v[0], v[1], v[2], v[3]});
+        qc.push_back(ushort4{c[0], c[1], c[2], c[3]});
+      }
+    }
+    rq[(size_t)r * (chunk + 1) + chunk] = (int)qv.size() - qoff[r];
+    for (int a = 0; a < m; ++a) {
+      const int q0 = at[a];
+      while (at[a] < cp[a + 1] && row[at[a]] < e) ++at[a];
+      if (at[a] == q0) continue;
+      acol.push_back(a);
+      abeg.push_back((int)er.size() - eoff[r]);
+      for (int q = q0; q < at[a]; ++q) {
+        er.push_back((uint16_t)(row[q] - b));
+        ev.push_back((float)val[q]);
+      }
+    }
+    qoff[r + 1] = (int)qv.size();
+    aoff[r + 1] = (int)acol.size();
+    eoff[r + 1] = (int)er.size();
+    d.xq_max = std::max(d.xq_max, qoff[r + 1] - qoff[r]);
+    d.xa_max = std::max(d.xa_max, aoff[r + 1] - aoff[r]);
+    d.xc_max = std::max(d.xc_max, eoff[r + 1] - eoff[r]);
+  }
+  int *d1, *d2, *d3, *d4, *d5, *d6;
+  float4* v1;
+  ushort4* c1;
+  uint16_t* r1;
+  float* v2;
+  TRY(upload(p, &d1, qoff));
+  TRY(upload(p, &d2, aoff));
+  TRY(upload(p, &d3, eoff));
+  TRY(upload(p, &d4, rq));
+  TRY(upload(p, &d5, acol));
+  TRY(upload(p, &d6, abeg));
+  TRY(upload(p, &v1, qv));
+  TRY(upload(p, &c1, qc));
+  TRY(upload(p, &r1, er));
+  TRY(upload(p, &v2, ev));
+  CUCHK(p, cudaStreamSynchronize(p->st));  // the host tables leave scope
+  d.xq_off = d1;
+  d.xa_off = d2;
+  d.xc_off = d3;
+  d.xr_q = d4;
+  d.xa_col = d5;
+  d.xa_beg = d6;
+  d.xr_v = v1;
+  d.xr_c = c1;
+  d.xc_r = r1;
+  d.xc_v = v2;
+  return CR_OK;
+}
+
 // Build the padded ELL layout and the PCG partition of one Laplacian.
 cr_status build_lap(cr_problem* p, const cr_csr& c, DevLap& L) {
   const int n = (int)c.n;
@@ -553,7 +711,7 @@ cr_status build_lap(cr_problem* p, const cr_csr& c, DevLap& L) {
   L.chunk = chunk;
   L.csize = cs;
   if (cs > 0) CUCHK(p, pcg_prepare(0, cs, pcg_smem_bytes(chunk, p->m)));
-  return CR_OK;
+  return build_push(p, rows, diag, L, p->push[&L == &p->Lx ? 1 : 0]);
 }
 
 // Grid-wide form of the multigrid PCG (cr_mg_grid.cu) on the hierarchy H.  It
@@ -1104,8 +1262,8 @@ PcgArgs pcg_args(cr_problem* p, int side, const double* b, double* x, int maxit,
   return a;
 }
 
-// Kernel choice: the register-resident cluster kernel while it applies (the
-// whole solve on chip); beyond it the grid-wide kernel, which measured as fast
+// Kernel choice: the register-resident cluster kernel (float64) or the pushing
+// one (float32) while it applies (the whole solve on chip); beyond it the grid-wide kernel, which measured as fast
 // as the generic cluster kernel at 45k voxels and twice as fast at 127k
 // (16 SMs against all of them); pcg_kernel = 1 / 2 force the generic cluster
 // or the grid-wide kernel.
@@ -1113,7 +1271,7 @@ bool use_grid_pcg(const cr_problem* p, int side, bool fp32) {
   const DevLap& L = side == 0 ? p->Ly : p->Lx;
   if (p->opt.pcg_kernel == 2 || L.csize == 0) return true;
   if (p->opt.pcg_kernel == 1) return false;
-  return pcg_reg_vpt(L, fp32) == 0;
+  return fp32 ? p->push[side].csize == 0 : pcg_reg_vpt(L) == 0;
 }
 
 // One Jacobi-PCG solve on the cluster-resident kernel, or on the grid-wide
@@ -1157,7 +1315,10 @@ cr_status run_pcg(cr_problem* p, int side, const double* b, double* x, int maxit
   }
   if (!use_grid_pcg(p, side, fp32)) {
     prof_begin(p, kph);
-    CUCHK(p, pcg_launch(pcg_args(p, side, b, x, maxit, tol, fp32), side, p->st));
+    if (fp32 && p->opt.pcg_kernel == 0)
+      CUCHK(p, pcg_push_launch(pcg_args(p, side, b, x, maxit, tol, fp32), p->push[side], side, p->st));
+    else
+      CUCHK(p, pcg_launch(pcg_args(p, side, b, x, maxit, tol, fp32), side, p->st));
     prof_end(p, kph);
     return CR_OK;
   }
@@ -2170,11 +2331,10 @@ cr_status cr_create(const cr_problem_desc* d_in, const cr_options* o, cr_problem
     CK(upload(p, &d_lp, lp));
     CK(upload(p, &d_lr, lr));
     CK(upload(p, &d_lv, lv));
-    std::vector<float> lvf(lv.begin(), lv.end()), rvf(rv.begin(), rv.end());
-    float *d_lvf, *d_rvf;
-    CK(upload(p, &d_lvf, lvf));
-    CK(upload(p, &d_rvf, rvf));
-    p->xl = DevXLocal{d_lp, d_lr, d_lv, d_rp, d_rc, d_rv, d_lvf, d_rvf};
+    p->xl = DevXLocal{d_lp, d_lr, d_lv, d_rp, d_rc, d_rv};
+    CK(build_push_x(p, p->push[1], cp, row, val, rp, rc, rv));
+    for (int side = 0; side < 2; ++side)
+      if (p->push[side].csize > 0 && !pcg_push_prepare(p->push[side], p->m, side)) p->push[side].csize = 0;
     if (p->mg[1].nlev > 0) {
       // |X_a|^2: the v side's mean data weight enters the multigrid shift
       std::vector<double> xn2(m, 0.0);

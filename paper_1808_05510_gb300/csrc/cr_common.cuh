@@ -73,8 +73,6 @@ struct DevXLocal {
   const int* xr_ptr = nullptr;   // [nx + 1]
   const int* xr_col = nullptr;
   const double* xr_val = nullptr;
-  const float* lx_valf = nullptr;  // float32 copies (mixed form)
-  const float* xr_valf = nullptr;
 };
 
 // Scalars the host reads back after a PCG solve.
@@ -111,7 +109,7 @@ struct PcgArgs {
   int maxit;
   PcgStat* stat;           // device
   int force_generic;       // 1: always use the shared/global-memory kernel
-  int fp32;                // 1: float32 vectors and arithmetic, float64 inner products and scalars
+  int fp32;                // 1: float32 vectors and arithmetic
 };
 
 // ---------------------------------------------------------------- cr_mg.cu
@@ -258,12 +256,42 @@ cudaError_t pcg_grid_launch(const PcgArgs& a, int side, const int* xc_ptr, const
                             double* work, double* part, double* ypart, double* yglob, unsigned* bar, int* err,
                             int nb, cudaStream_t st);
 
+// ---------------------------------------------------------------- cr_pcg_push.cu
+// Tables of the float32 cluster PCG, which pushes values to the CTAs that need
+// them.  CTA r numbers its own rows 0 .. chunk-1 and the rows within two hops of
+// them chunk, chunk + 1, ... in row order; ext - 1 is a zero word (missing
+// neighbour).
+struct DevPush {
+  int csize = 0;  // CTAs of the cluster (0: not available)
+  int chunk = 0, ext = 0, hmax = 0, P = 0;
+  const uint4* own = nullptr;      // [n] the row's six neighbours as 16-bit pairs (x, y, z)
+  const int* hcnt = nullptr;       // [csize] rows of other CTAs next to this one's
+  const uint4* hn = nullptr;       // [csize * hmax] their neighbours and their own number (w)
+  const double* hdiag = nullptr;   // [csize * hmax] L_ii
+  const uint32_t* push = nullptr;  // [csize][P][chunk] (receiving CTA << 16) | number there, or ~0
+  // v side (xq_max >= 0): each CTA's rows of X padded to quads (offsets xr_q per row), and its
+  // part of the columns with an entry in it (xa_col, first entry xa_beg, rows xc_r, values xc_v)
+  int xq_max = -1, xa_max = 0, xc_max = 0;
+  int x_smem = 0;  // the v side's part is copied to shared memory
+  const int *xq_off = nullptr, *xa_off = nullptr, *xc_off = nullptr;  // [csize + 1]
+  const int* xr_q = nullptr;
+  const float4* xr_v = nullptr;
+  const ushort4* xr_c = nullptr;
+  const int *xa_col = nullptr, *xa_beg = nullptr;
+  const uint16_t* xc_r = nullptr;
+  const float* xc_v = nullptr;
+};
+// Sets d.x_smem; false where the kernel does not fit.
+bool pcg_push_prepare(DevPush& d, int m, int side);
+// Solves from x = 0 in float32; a.dinv and (u side) a.omt hold the Jacobi inverse diagonal and omega.
+cudaError_t pcg_push_launch(const PcgArgs& a, const DevPush& d, int side, cudaStream_t st);
+
 // ---------------------------------------------------------------- cr_pcg.cu
 cudaError_t pcg_launch(const PcgArgs& a, int data_kind, cudaStream_t st);
 cudaError_t pcg_prepare(int data_kind, int csize, size_t smem_bytes);
 size_t pcg_smem_bytes(int chunk, int m);
-// rows per thread of the register-resident cluster kernel for this operator, 0 if it does not apply
-int pcg_reg_vpt(const DevLap& L, bool fp32);
+// rows per thread of the register-resident float64 cluster kernel for this operator, 0 if it does not apply
+int pcg_reg_vpt(const DevLap& L);
 bool pcg_cluster_ok(int csize, size_t smem_bytes);
 // y = (L + shift I) x
 void lap_apply(const DevLap& L, const double* x, double* y, double shift, cudaStream_t st);
