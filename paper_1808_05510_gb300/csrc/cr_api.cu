@@ -532,7 +532,6 @@ cr_status build_push(cr_problem* p, const std::vector<std::vector<std::pair<int,
   TRY(upload(p, &d3, hcnt));
   TRY(upload(p, &d4, hd));
   TRY(upload(p, &d5, push));
-  CUCHK(p, cudaStreamSynchronize(p->st));  // the host tables leave scope
   d.own = d1;
   d.hn = d2;
   d.hcnt = d3;
@@ -606,7 +605,6 @@ cr_status build_push_x(cr_problem* p, DevPush& d, const std::vector<int>& cp, co
   TRY(upload(p, &c1, qc));
   TRY(upload(p, &r1, er));
   TRY(upload(p, &v2, ev));
-  CUCHK(p, cudaStreamSynchronize(p->st));  // the host tables leave scope
   d.xq_off = d1;
   d.xa_off = d2;
   d.xc_off = d3;
@@ -694,6 +692,22 @@ cr_status build_lap(cr_problem* p, const cr_csr& c, DevLap& L) {
       nbrp[k * n + i] = ((jj / chunk) << 24) | (jj % chunk);
       if (!unit) offw[k * n + i] = rows[i][k].second;
     }
+  // 16-bit distances for the grid-wide PCG, wherever it may run
+  bool near16 = unit && K <= 6 && (cs == 0 || chunk > 2 * kPcgThreads || p->opt.pcg_kernel == 2);
+  std::vector<uint32_t> nbr16(near16 ? (size_t)3 * n : 0, 0u);
+  for (int i = 0; near16 && i < n; ++i) {
+    if (diag[i] != (double)rows[i].size()) near16 = false;
+    for (size_t k = 0; k < rows[i].size(); ++k) {
+      const int d = rows[i][k].first - i;
+      if (d > 32767 || d < -32767) near16 = false;
+      nbr16[(k / 2) * n + i] |= (uint32_t)(uint16_t)(int16_t)d << (16 * (k & 1));
+    }
+  }
+  if (near16) {
+    uint32_t* d16 = nullptr;
+    TRY(upload(p, &d16, nbr16));
+    L.nbr16 = d16;
+  }
   int *dn = nullptr, *dnp = nullptr;
   double *dd = nullptr, *dl2 = nullptr, *dw = nullptr;
   TRY(upload(p, &dn, nbr));
@@ -800,7 +814,6 @@ cr_status build_mg_grid(cr_problem* p, const DevLap& L, const cr_mg::Hierarchy& 
     TRY(upload(p, &v4, T.a));
     TRY(upload(p, &v5, T.b));
     TRY(upload(p, &v6, T.c));
-    CUCHK(p, cudaStreamSynchronize(p->st));  // S and T leave scope
     W.srp = d1;
     W.sci = d2;
     W.sp = v1;
@@ -1078,12 +1091,12 @@ cr_status build_mg(cr_problem* p, const cr_csr& c, const DevLap& L, DevMg& g) {
 // then w <- w / |w|.  Returns |w_after| / |w_before| (0 if w was zero).
 cr_status cgs2(cr_problem* p, int n, const double* Q, int64_t ldq, int nq, double* w, double* ratio) {
   cudaStream_t st = p->st;
-  dot(n, w, w, p->ds + DS_NB, st);
+  dot(n, w, w, p->ds + DS_NB, p->ws, st);
   for (int pass = 0; pass < 2 && nq > 0; ++pass) {
     gemv_t(n, nq, Q, ldq, w, p->cvec, 1, 1.0, 0.0, st);
     gemv_n(n, nq, Q, ldq, p->cvec, 1, w, -1.0, 1.0, st);
   }
-  dot(n, w, w, p->ds + DS_NA, st);
+  dot(n, w, w, p->ds + DS_NA, p->ws, st);
   TRY(readback(p, DS_NB, 2, false));
   const double nb = p->hs->ds[DS_NB], na = p->hs->ds[DS_NA];
   *ratio = nb > 0.0 ? std::sqrt(na / nb) : 0.0;
@@ -1121,8 +1134,8 @@ void residual_t_times(cr_problem* p, const double* uu, double* out) {
 void prep_u(cr_problem* p, const double* vv) {
   cudaStream_t st = p->st;
   lap_apply(p->Lx, vv, p->tmpx, 0.0, st);
-  dot(p->nx, vv, p->tmpx, p->coef + 0, st);
-  dot(p->nx, p->tmpx, p->tmpx, p->coef + 1, st);
+  dot(p->nx, vv, p->tmpx, p->coef + 0, p->ws, st);
+  dot(p->nx, p->tmpx, p->tmpx, p->coef + 1, p->ws, st);
   spmv_xt(p->m, p->xc_ptr, p->xc_row, p->xc_val, vv, p->xi, 1, st);
 }
 
@@ -1130,8 +1143,8 @@ void prep_u(cr_problem* p, const double* vv) {
 void prep_v(cr_problem* p, const double* uu) {
   cudaStream_t st = p->st;
   lap_apply(p->Ly, uu, p->tmpy, 0.0, st);
-  dot(p->ny, uu, p->tmpy, p->coef + 2, st);
-  dot(p->ny, p->tmpy, p->tmpy, p->coef + 3, st);
+  dot(p->ny, uu, p->tmpy, p->coef + 2, p->ws, st);
+  dot(p->ny, p->tmpy, p->tmpy, p->coef + 3, p->ws, st);
   omega_sq_dots(p->ny, p->m, p->Om, p->ny, uu, p->svec, st);
 }
 
@@ -1160,11 +1173,11 @@ cr_status fcg_learned(cr_problem* p, int side, const double* b, double* x) {
   fcg_apply(L, p->lam, coef, side, p->pomt, p->xl, p->xc_ptr, p->xc_row, p->xc_val, p->m, p->svec, p->fc_y, x, t, q,
             st);
   mat_axpby(n, 1, 1.0, b, n, -1.0, q, n, r, n, st);  // r = b - A x
-  dot(n, b, b, sc + 5, st);
+  dot(n, b, b, sc + 5, p->ws, st);
   fcg_precond(n, p->box[side], p->pdinv, r, sc + 4, p->net_in, p->net_V, p->net, p->net_out, z, st);
   copy(n, z, pv, st);
-  dot(n, r, z, sc + 0, st);
-  dot(n, r, r, sc + 2, st);
+  dot(n, r, z, sc + 0, p->ws, st);
+  dot(n, r, r, sc + 2, p->ws, st);
   TRY(readback(p, DS_FCG, 6, false));
   const double bb = p->hs->ds[DS_FCG + 5];
   const double tol2 = tol * tol * bb;
@@ -1176,14 +1189,14 @@ cr_status fcg_learned(cr_problem* p, int side, const double* b, double* x) {
   while (bb > 0.0 && rr > tol2 && k < cap) {
     fcg_apply(L, p->lam, coef, side, p->pomt, p->xl, p->xc_ptr, p->xc_row, p->xc_val, p->m, p->svec, p->fc_y, pv, t,
               q, st);
-    dot(n, pv, q, sc + 1, st);
+    dot(n, pv, q, sc + 1, p->ws, st);
     fcg_update_xr(n, x, r, rold, pv, q, sc, st);
-    dot(n, r, r, sc + 2, st);
+    dot(n, r, r, sc + 2, p->ws, st);
     fcg_precond(n, p->box[side], p->pdinv, r, sc + 4, p->net_in, p->net_V, p->net, p->net_out, z, st);
     fcg_diff(n, r, rold, dd, st);
-    dot(n, z, dd, sc + 3, st);
+    dot(n, z, dd, sc + 3, p->ws, st);
     fcg_update_p(n, pv, z, sc, st);
-    dot(n, r, z, sc + 0, st);
+    dot(n, r, z, sc + 0, p->ws, st);
     ++k;
     if (k < 8 || (k % 4) == 0) {
       TRY(readback(p, DS_FCG, 3, false));
@@ -1336,7 +1349,7 @@ cr_status run_pcg(cr_problem* p, int side, const double* b, double* x, int maxit
     TRY(dalloc(p, &p->pg_err, 1));
   }
   const DevLap& L = side == 0 ? p->Ly : p->Lx;
-  const int nb = pcg_grid_blocks(fp32, p->m, L.K);
+  const int nb = pcg_grid_blocks(fp32, p->m, L);
   if (nb < 1) return fail(p, CR_ECUDA, "the grid-wide PCG cannot be launched on this device");
   const double* coef = p->coef + (side == 0 ? 0 : 2);
   fcg_jacobi_diag(L, p->lam, coef, side, p->m, p->Om, p->ny, p->xi, p->xl, p->svec, p->pomt, p->pdinv, p->st);
@@ -1378,7 +1391,7 @@ cr_status launch_pcg_mixed(cr_problem* p, int side, const double* b, double* x, 
   const double tol = p->opt.pcg_tol;
   prof_begin(p, side == 0 ? CR_PHASE_PCG_U : CR_PHASE_PCG_V);
   fcg_jacobi_diag(L, p->lam, coef, side, p->m, p->Om, p->ny, p->xi, p->xl, p->svec, p->pomt, p->pdinv, st);
-  dot(n, b, b, sc + 0, st);
+  dot(n, b, b, sc + 0, p->ws, st);
   PcgStat hs{0, 0, 0.0, 0.0};
   int total = 0;
   double rr_prev = INFINITY;
@@ -1386,7 +1399,7 @@ cr_status launch_pcg_mixed(cr_problem* p, int side, const double* b, double* x, 
     fcg_apply(L, p->lam, coef, side, p->pomt, p->xl, p->xc_ptr, p->xc_row, p->xc_val, p->m, p->svec, p->fc_y, x,
               p->fc_t, q, st);
     mat_axpby(n, 1, 1.0, b, n, -1.0, q, n, r, n, st);  // r = b - A x (float64)
-    dot(n, r, r, sc + 1, st);
+    dot(n, r, r, sc + 1, p->ws, st);
     TRY(readback(p, DS_REF, 2, false));
     const double bb = p->hs->ds[DS_REF], rr = p->hs->ds[DS_REF + 1];
     hs.bnorm = std::sqrt(bb);
@@ -2016,7 +2029,7 @@ cr_status do_rank_one(cr_problem* p, cr_rank1_info* info) {
   // ALS start vector: v0 = R_j^T 1 / |R_j^T 1|
   fill(ny, 1.0, p->tmpy, st);
   residual_t_times(p, p->tmpy, p->v);
-  dot(nx, p->v, p->v, p->ds + DS_V0, st);
+  dot(nx, p->v, p->v, p->ds + DS_V0, p->ws, st);
   TRY(readback(p, DS_V0, 1, false));
   const double v0n2 = p->hs->ds[DS_V0];
   if (v0n2 > 1e-300 * p->Dnorm * p->Dnorm && std::isfinite(v0n2)) {
@@ -2055,13 +2068,13 @@ cr_status do_rank_one(cr_problem* p, cr_rank1_info* info) {
     prof_end(p, CR_PHASE_RHS);
     TRY(launch_pcg(p, 0, p->rhs_u, p->uhat));
     prof_begin(p, CR_PHASE_RHS);
-    dot(ny, p->uhat, p->uhat, p->ds + DS_UN2, st);
+    dot(ny, p->uhat, p->uhat, p->ds + DS_UN2, p->ws, st);
     scale_by_inv_norm(ny, p->uhat, p->ds + DS_UN2, p->u, st);
     prep_v(p, p->u);
     residual_t_times(p, p->u, p->rhs_v);
     prof_end(p, CR_PHASE_RHS);
     TRY(launch_pcg(p, 1, p->rhs_v, p->vhat));
-    dot(nx, p->vhat, p->vhat, p->ds + DS_VN2, st);
+    dot(nx, p->vhat, p->vhat, p->ds + DS_VN2, p->ws, st);
     scale_by_inv_norm(nx, p->vhat, p->ds + DS_VN2, p->v, st);
     TRY(readback(p, 0, 2, true));
     const PcgStat* s = p->hs->stat;
@@ -2459,7 +2472,7 @@ cr_status cr_create(const cr_problem_desc* d_in, const cr_options* o, cr_problem
   CK(dalloc(p, &p->gram, (size_t)m * m));
   CK(dalloc(p, &p->tmat, (size_t)m * m));
   p->ws_elems = std::max<size_t>((size_t)8 * p->ldcp * p->ldm, (size_t)16 * (3 * rc + m) * m);
-  p->ws_elems = std::max<size_t>(p->ws_elems, (size_t)16 * r2);
+  p->ws_elems = std::max<size_t>(std::max<size_t>(p->ws_elems, (size_t)16 * r2), 1024);
   CK(dalloc(p, &p->ws, p->ws_elems));
   // right residual basis: X first (host Gram-Schmidt twice, columns in X's span rejected)
   {

@@ -56,6 +56,9 @@ struct DevLap {
   int K = 0;                     // slots per row (padded entries are -1)
   const int* nbr = nullptr;      // [K * n] global column, -1 = none
   const int* nbrp = nullptr;     // [K * n] packed (rank, local), -1 = none
+  // grid-wide PCG, unit-weight graph Laplacians (L_ii the number of neighbours, at most six, none
+  // further than 32,767 rows away): six signed 16-bit distances per row, two to a word, 0 = none
+  const uint32_t* nbr16 = nullptr;  // [3 * n]
   const double* offw = nullptr;  // [K * n] or nullptr (unit Laplacian)
   const double* diag = nullptr;  // [n]  L_ii
   const double* l2diag = nullptr;// [n]  (L^2)_ii = L_ii^2 + sum_k L_ik^2
@@ -246,10 +249,10 @@ cudaError_t mg_grid_launch(const PcgArgs& a, const DevMg& g, const DevMgGrid& d,
 // ---------------------------------------------------------------- cr_pcg_grid.cu
 // Grid-wide PCG (vectors in HBM, all SMs) for grids the register-resident cluster kernel does not take.
 // Blocks of the cooperative launch (0: cannot run) and work doubles needed.
-int pcg_grid_blocks(bool fp32, int m, int K);
+int pcg_grid_blocks(bool fp32, int m, const DevLap& L);
 size_t pcg_grid_work_elems(int n);
 // Solves the system of `a` (side 0: Eq. ALS_linsys, 1: Eq. ALS_linsys_v) with
-// a.dinv, a.omt precomputed in float64 (fcg_jacobi_diag).  work: 9n doubles;
+// a.dinv, a.omt precomputed in float64 (fcg_jacobi_diag).  work: pcg_grid_work_elems doubles;
 // part: nb*4, ypart: nb*m, yglob: m doubles; bar: 2 unsigned; err: 1 int.
 // a.stat receives iterations and status (3 = grid barrier timed out).
 cudaError_t pcg_grid_launch(const PcgArgs& a, int side, const int* xc_ptr, const int* xc_row, const double* xc_val,
@@ -315,8 +318,8 @@ void gemv_t(int n, int k, const double* A, int64_t lda, const double* w, double*
 // y[i] = beta * y[i] + alpha * sum_p A[i + p*lda] * c[p*cstride]
 void gemv_n(int n, int k, const double* A, int64_t lda, const double* c, int64_t cstride, double* y,
             double alpha, double beta, cudaStream_t st);
-// out = alpha * sum_i x[i] * y[i] into *out (single deterministic reduction)
-void dot(int n, const double* x, const double* y, double* out, cudaStream_t st);
+// *out = sum_i x[i] * y[i] (deterministic; ws: 1,024 doubles of work, or null for one block)
+void dot(int n, const double* x, const double* y, double* out, double* ws, cudaStream_t st);
 // out[a * ostride] = sum over the nonzeros of column a of X (CSC) of X_ka * v[k]
 void spmv_xt(int m, const int* colptr, const int* row, const double* val, const double* v, double* out,
              int64_t ostride, cudaStream_t st);

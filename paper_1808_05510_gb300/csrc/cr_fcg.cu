@@ -139,7 +139,7 @@ void fcg_precond(int n, const int* box, const double* dinv, const double* r, dou
   }
   count_launch();
   dinv_r_kernel<<<nb256(n), 256, 0, st>>>(n, dinv, r, z);
-  dot(n, z, z, s2, st);
+  dot(n, z, z, s2, nullptr, st);
   cudaMemsetAsync(in, 0, sizeof(float) * 2 * V, st);
   count_launch();
   net_input_kernel<<<nb256(n), 256, 0, st>>>(n, box, dinv, r, s2, in, V);

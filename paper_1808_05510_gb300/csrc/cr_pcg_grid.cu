@@ -7,41 +7,48 @@
 // sweeps separated by a bounded grid barrier (the v side adds one short
 // sweep: block a adds column a of the per-block partial X^T p, so that every
 // block then reads y = s o X^T p for its data term X diag(s) X^T p):
-//   A2a  p = D^-1 r + beta p_old and t = (L + cI) p.  Row i needs p on its
-//        one-hop neighbourhood, recomputed from r and p_old (p is double
+//   A2a  p = z + beta p_old (z = D^-1 r) and t = (L + cI) p.  Row i needs p on
+//        its one-hop neighbourhood, recomputed from z and p_old (p is double
 //        buffered), so no barrier separates the p update from the stencil;
 //   A2b  q = lam ((L + cI) t + e p) + data(p), and the block's partial <p, q>;
-//   B    alpha = rho / <p, q>, x += alpha p, r -= alpha q, and the partials
-//        of rho' = <r, D^-1 r> and |r|^2.
+//   B    alpha = rho / <p, q>, x += alpha p, r -= alpha q, z = D^-1 r, and the
+//        partials of rho' = <r, z> and |r|^2; four rows per thread and load.
 // The operator holds (L + cI)^2; splitting it through t keeps every row's
 // loads one hop deep, with the neighbour indices fetched before the values.
 // Reads of data that other blocks wrote before the last grid barrier are
-// ordinary (L1-cached) loads: the barrier's acquire fence at GPU scope, taken
-// before the block passes its CTA barrier, makes those writes visible (the
-// cooperative-groups grid synchronisation pattern), and adjacent rows share
-// most of their neighbourhoods in L1.
+// ordinary (L1-cached) loads: the barrier's acquire at GPU scope, taken before
+// the block passes its CTA barrier, makes those writes visible, and adjacent
+// rows share most of their neighbourhoods in L1.
 // Every block adds the per-block partial sums itself, in one fixed order, so
 // all blocks hold bit-identical scalars and take identical decisions.
 // T = float: float32 vectors and arithmetic with double-float (two-float)
 // accumulation of the inner products; T = double: float64 throughout (on
 // GB300 the float64 form is bound by float64 arithmetic, not by HBM).
-// Bytes per row and iteration in float32 (unit-weight Laplacian, K = 6):
-// A2a reads r, p_old, D^-1, L_ii, the neighbour table and writes p, t (48 B);
-// A2b reads t, p, L_ii, omega, the table and writes q (44 B); B reads x, p, r,
-// q, D^-1 and writes x, r (28 B): 120 B, against the 64 B of the two-sweep
-// minimum (r, x, p, q once each way, D^-1, omega, the table): the table and
-// L_ii are read twice and t makes one round trip.
+// Neighbour tables: a unit-weight graph Laplacian with at most six neighbours
+// per row, none further than 32,767 rows away, stores the six distances as
+// 16-bit integers (12 B per row instead of 24 B, and L_ii is their count);
+// every other matrix keeps 32-bit indices, weights and L_ii.
+// Bytes per row and iteration in float32 with the 16-bit table: A2a reads z,
+// p_old, the table and writes p, t (28 B); A2b reads t, p, omega, the table and
+// writes q (28 B); B reads x, p, r, q, D^-1 and writes x, r, z (32 B): 88 B
+// (120 B with 32-bit indices, L_ii, and z formed from r and D^-1 at every
+// neighbour, which also took seven gathers more).
+// Measured with it against that form (us per iteration, ellipsoidal shells):
+// float32 200,160 voxels 38 -> 18, 1.0M 61 -> 26, 3.0M 158 -> 69 (3.8 TB/s of the
+// 88 B); float64 1.0M 102 -> 75, 3.0M 267 -> 201.
 #include <algorithm>
 
 #include "cr_common.cuh"
 #include "cr_df.cuh"
+#include "cr_grid_bar.cuh"
 
 namespace cr {
 
 namespace {
 
-constexpr int kGThreads = 512;
-constexpr long long kGridSpin = 1ll << 24;
+// One CTA of 1,024 threads per SM with the 16-bit table, at most two of 512 with the general one:
+// (every further CTA lengthens the barriers and the sums behind them).
+constexpr int kGThreads16 = 1024, kGThreads = 512;
 
 struct GridPcg {
   DevLap L;
@@ -68,11 +75,13 @@ struct GridPcg {
   void* ts;            // [n] T: t = (L + cI) p
   void* ds;            // [n] T: D^-1
   void* os;            // [n] T: omega (u side)
-  void* gs;            // [n] T: L_ii
+  void* gs;            // [n] T: L_ii (32-bit table)
+  void* zs;            // [n] T: z = D^-1 r
+  const uint32_t* idx; // [3 * n] six 16-bit neighbour distances per row (0: none), or null
   double* part;        // [nb * kParts] per-block partial sums
   double* ypart;       // v side [nb * m] per-block partial X^T p
   double* yglob;       // v side [m] y = s o X^T p
-  unsigned* bar;       // [2] barrier counter, generation
+  unsigned* bar;       // barrier counter
   int* err;            // barrier timeout flag
   int nb, chunk;
   double tol;
@@ -82,41 +91,6 @@ struct GridPcg {
 
 constexpr int kParts = 4;  // (p,q), rho, |r|^2, |b|^2
 
-__device__ __forceinline__ bool grid_sync(const GridPcg& a) {
-  __syncthreads();
-  __shared__ int ok;
-  if (threadIdx.x == 0) {
-    volatile unsigned* gen = a.bar + 1;
-    const unsigned g = *gen;
-    __threadfence();
-    const unsigned arrived = atomicAdd(a.bar, 1u) + 1u;
-    int good = 1;
-    if (arrived == (unsigned)a.nb) {
-      atomicExch(a.bar, 0u);
-      __threadfence();
-      atomicAdd(a.bar + 1, 1u);
-    } else {
-      long long spins = 0;
-      while (*gen == g) {
-        if (*(volatile int*)a.err) {
-          good = 0;
-          break;
-        }
-        if (++spins > kGridSpin) {
-          atomicExch(a.err, 1);
-          good = 0;
-          break;
-        }
-        __nanosleep(32);
-      }
-    }
-    __threadfence();
-    ok = good && !*(volatile int*)a.err;
-  }
-  __syncthreads();
-  return ok;
-}
-
 // Accumulator of an inner product: double-float for float32 vectors, double otherwise.
 template <class T>
 struct Acc;
@@ -124,97 +98,173 @@ template <>
 struct Acc<float> {
   DF v{0.f, 0.f};
   __device__ void add(float a, float b) { v = df_add(v, df_prod(a, b)); }
-  __device__ double get() const { return (double)v.hi + (double)v.lo; }
 };
 template <>
 struct Acc<double> {
   double v = 0.0;
   __device__ void add(double a, double b) { v = fma(a, b, v); }
-  __device__ double get() const { return v; }
 };
 
-// Block sum of NV doubles in a fixed tree order; result in out[] of thread 0.
+// four consecutive rows of a vector
+__device__ __forceinline__ void ld4(float (&v)[4], const float* p) {
+  const float4 q = *reinterpret_cast<const float4*>(p);
+  v[0] = q.x;
+  v[1] = q.y;
+  v[2] = q.z;
+  v[3] = q.w;
+}
+__device__ __forceinline__ void ld4(double (&v)[4], const double* p) {
+  const double2 a = *reinterpret_cast<const double2*>(p), b = *reinterpret_cast<const double2*>(p + 2);
+  v[0] = a.x;
+  v[1] = a.y;
+  v[2] = b.x;
+  v[3] = b.y;
+}
+__device__ __forceinline__ void st4(float* p, const float (&v)[4]) {
+  *reinterpret_cast<float4*>(p) = float4{v[0], v[1], v[2], v[3]};
+}
+__device__ __forceinline__ void st4(double* p, const double (&v)[4]) {
+  *reinterpret_cast<double2*>(p) = double2{v[0], v[1]};
+  *reinterpret_cast<double2*>(p + 2) = double2{v[2], v[3]};
+}
+
+// Block sums of NV accumulators in a fixed tree order; results in out[] of thread 0.
+// Float64 adds take 16 issue cycles a warp, so a shuffle tree over every warp costs
+// 2,560 of them per value at 1,024 threads: the double-float form sums its warps in
+// float32, the float64 form lets 128 threads add eight values each from shared memory.
 template <int NV>
-__device__ __forceinline__ void block_reduce(double (&v)[NV], double* out) {
-  __shared__ double sh[kGThreads / 32][NV];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+__device__ __forceinline__ void block_reduce(Acc<float> (&v)[NV], double* out) {
+  __shared__ double sh[32][NV];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
-    double t = v[k];
+    const DF t = warp_sum_df(v[k].v);
+    if (lane == 0) sh[w][k] = (double)t.hi + (double)t.lo;
+  }
+  __syncthreads();
+  if (w < NV) {
+    double t = lane < nw ? sh[lane][w] : 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) sh[w][k] = t;
+    if (lane == 0) out[w] = t;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
+}
+template <int NV>
+__device__ __forceinline__ void block_reduce(Acc<double> (&v)[NV], double* out) {
+  __shared__ double sh[NV][kGThreads16], sw[4][NV];
+  const int nt = blockDim.x;  // 512 or 1,024
+#pragma unroll
+  for (int k = 0; k < NV; ++k) sh[k][threadIdx.x] = v[k].v;
+  __syncthreads();
+  if (threadIdx.x < 128) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
-      double t = 0.0;
-      for (int q = 0; q < kGThreads / 32; ++q) t += sh[q][k];
-      out[k] = t;
+      double q[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) q[u] = threadIdx.x + 128 * u < nt ? sh[k][threadIdx.x + 128 * u] : 0.0;
+      double t = ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+      if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5][k] = t;
     }
   }
   __syncthreads();
+  if (threadIdx.x < NV) out[threadIdx.x] = ((sw[0][threadIdx.x] + sw[1][threadIdx.x]) + sw[2][threadIdx.x]) + sw[3][threadIdx.x];
+  __syncthreads();
 }
 
-// Sum of part[b * stride + k] over all blocks b, in the same order in every block.
-__device__ __forceinline__ double sum_parts(const double* part, int nb, int stride, int k) {
-  __shared__ double sh[kGThreads / 32];
-  __shared__ double res;
-  double t = 0.0;
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) t += __ldcg(part + (size_t)b * stride + k);
+// Sums of part[b * kParts + k] over all blocks b, k < NV, in the same order in every block.
+template <int NV>
+__device__ __forceinline__ void sum_parts(const double* part, int nb, int first, double (&out)[NV]) {
+  __shared__ double res[NV];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w < NV) {
+    double t = 0.0;
+    for (int b = lane; b < nb; b += 8 * 32) {
+      double v[8];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-  if (lane == 0) sh[w] = t;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double u = 0.0;
-    for (int q = 0; q < kGThreads / 32; ++q) u += sh[q];
-    res = u;
-  }
-  __syncthreads();
-  const double out = res;
-  __syncthreads();
-  return out;
-}
-
-// Neighbour indices of row i (KM slots; -1 = none).  The table is never
-// written during the solve: read-only path.
-template <int KM>
-__device__ __forceinline__ void load_nbrs(const DevLap& L, int i, int (&q)[KM]) {
-#pragma unroll
-  for (int sl = 0; sl < KM; ++sl) q[sl] = sl < L.K ? __ldg(L.nbr + (size_t)sl * L.n + i) : -1;
-}
-
-// Row i of (L + cI) v with the neighbour indices already loaded; v(l) from the functor.
-template <class T, int KM, class VF>
-__device__ __forceinline__ T shifted_row(const DevLap& L, const T* gs, int i, const int (&q)[KM], T c,
-                                         const VF& v) {
-  T acc = (gs[i] + c) * v(i);
-#pragma unroll
-  for (int sl = 0; sl < KM; ++sl) {
-    if (q[sl] >= 0) {
-      const T w = L.offw ? (T)__ldg(L.offw + (size_t)sl * L.n + i) : (T)-1;
-      acc = fma(w, v(q[sl]), acc);
+      for (int u = 0; u < 8; ++u) v[u] = b + 32 * u < nb ? __ldcg(part + (size_t)(b + 32 * u) * kParts + first + w) : 0.0;
+      t += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) res[w] = t;
   }
-  return acc;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NV; ++k) out[k] = res[k];
+  __syncthreads();
 }
 
-// f(i, q) over the block's rows, two rows per thread and step: both rows'
-// neighbour indices are loaded before either row's values, so each thread
-// keeps two rows' loads in flight (the sweeps are bound by memory latency).
-template <int KM, class F>
-__device__ __forceinline__ void for_rows2(const DevLap& L, int lo, int hi, const F& f) {
+// Neighbours of row i (KM slots; -1 = none).  The table is never written during
+// the solve: read-only path.  Returns L_ii where the table holds 16-bit distances.
+template <bool F16, int KM>
+__device__ __forceinline__ int load_nbrs(const GridPcg& a, int i, int (&q)[KM]) {
+  if constexpr (F16) {
+    const int n = a.L.n;
+    int deg = 0;
+    uint32_t w[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) w[k] = __ldg(a.idx + (size_t)k * n + i);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const int d = (int)(int16_t)(k & 1 ? w[k >> 1] >> 16 : w[k >> 1] & 0xFFFFu);
+      q[k] = d ? i + d : -1;
+      deg += d ? 1 : 0;
+    }
+    return deg;
+  } else {
+#pragma unroll
+    for (int sl = 0; sl < KM; ++sl) q[sl] = sl < a.L.K ? __ldg(a.L.nbr + (size_t)sl * a.L.n + i) : -1;
+    return 0;
+  }
+}
+
+// Row i of (L + cI) v with the neighbours already loaded; vi = v(i), v(l) from the functor.
+template <class T, bool F16, int KM, class VF>
+__device__ __forceinline__ T shifted_row(const GridPcg& a, const T* gs, int i, const int (&q)[KM], int deg, T c, T vi,
+                                         const VF& v) {
+  if constexpr (F16) {
+    T w[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) w[k] = q[k] >= 0 ? v(q[k]) : (T)0;
+    return ((T)deg + c) * vi - (((w[0] + w[1]) + (w[2] + w[3])) + (w[4] + w[5]));
+  } else {
+    T acc = (gs[i] + c) * vi;
+#pragma unroll
+    for (int sl = 0; sl < KM; ++sl) {
+      if (q[sl] >= 0) {
+        const T w = a.L.offw ? (T)__ldg(a.L.offw + (size_t)sl * a.L.n + i) : (T)-1;
+        acc = fma(w, v(q[sl]), acc);
+      }
+    }
+    return acc;
+  }
+}
+
+// f(i, q, deg) over the block's rows.  With the general table two rows per thread
+// and step, both rows' neighbours loaded before either row's values, so that each
+// thread keeps two rows' loads in flight (the sweeps are bound by memory latency);
+// with the 16-bit table one row, which leaves registers for twice the threads.
+template <bool F16, int KM, class F>
+__device__ __forceinline__ void for_rows(const GridPcg& a, int lo, int hi, const F& f) {
   const int bd = blockDim.x;
-  for (int i0 = lo + threadIdx.x; i0 < hi; i0 += 2 * bd) {
-    const int i1 = i0 + bd;
-    int q0[KM], q1[KM];
-    load_nbrs<KM>(L, i0, q0);
-    if (i1 < hi) load_nbrs<KM>(L, i1, q1);
-    f(i0, q0);
-    if (i1 < hi) f(i1, q1);
+  if constexpr (F16) {
+    for (int i = lo + threadIdx.x; i < hi; i += bd) {
+      int q[KM];
+      const int deg = load_nbrs<F16, KM>(a, i, q);
+      f(i, q, deg);
+    }
+  } else {
+    for (int i0 = lo + threadIdx.x; i0 < hi; i0 += 2 * bd) {
+      const int i1 = i0 + bd;
+      int q0[KM], q1[KM];
+      load_nbrs<F16, KM>(a, i0, q0);
+      if (i1 < hi) load_nbrs<F16, KM>(a, i1, q1);
+      f(i0, q0, 0);
+      if (i1 < hi) f(i1, q1, 0);
+    }
   }
 }
 
@@ -250,7 +300,7 @@ __device__ __forceinline__ void xt_partial(const GridPcg& a, int lo, int hi, con
 // Second stage of the v side's X^T v: block a adds column a of the per-block
 // partials (fixed order) and stores y_a = s_a (X^T v)_a.
 __device__ __forceinline__ void reduce_y_global(const GridPcg& a) {
-  __shared__ double sh[kGThreads / 32];
+  __shared__ double sh[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int col = blockIdx.x; col < a.m; col += a.nb) {
     double t = 0.0;
@@ -261,7 +311,7 @@ __device__ __forceinline__ void reduce_y_global(const GridPcg& a) {
     __syncthreads();
     if (threadIdx.x == 0) {
       double u = 0.0;
-      for (int q = 0; q < kGThreads / 32; ++q) u += sh[q];
+      for (int q = 0; q < (int)(blockDim.x >> 5); ++q) u += sh[q];
       a.yglob[col] = a.s[col] * u;
     }
     __syncthreads();
@@ -283,8 +333,8 @@ __device__ __forceinline__ T data_row(const GridPcg& a, const T* om, const doubl
   return acc;
 }
 
-template <class T, int KM>
-__global__ void __launch_bounds__(kGThreads) pcg_grid_kernel(const GridPcg a) {
+template <class T, int KM, bool F16>
+__global__ void __launch_bounds__(F16 ? kGThreads16 : kGThreads, 1) pcg_grid_kernel(const GridPcg a) {
   extern __shared__ double ys[];  // v side: y = s o (X^T v), m entries
   __shared__ double red[kParts];
   T* xs = (T*)a.xs;
@@ -294,6 +344,8 @@ __global__ void __launch_bounds__(kGThreads) pcg_grid_kernel(const GridPcg a) {
   T* dv = (T*)a.ds;
   T* om = (T*)a.os;
   T* gs = (T*)a.gs;
+  T* zs = (T*)a.zs;
+  GridBar bar = grid_bar(a.bar, a.err);
   const int n = a.L.n;
   const int lo = min(n, blockIdx.x * a.chunk), hi = min(n, lo + a.chunk);
   const double cd = a.coef[0], dd = a.coef[1];
@@ -305,37 +357,40 @@ __global__ void __launch_bounds__(kGThreads) pcg_grid_kernel(const GridPcg a) {
   for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
     xs[i] = (T)a.x[i];
     dv[i] = (T)a.dinv64[i];
-    gs[i] = (T)a.L.diag[i];
+    if (!F16) gs[i] = (T)a.L.diag[i];
     if (a.side == 0) om[i] = (T)a.omt64[i];
   }
-  if (!grid_sync(a)) goto done;
+  if (!grid_bar_sync(bar)) goto done;
   // ---- t = (L + cI) x0; v side partial X^T x0
   {
     auto xv = [&](int l) { return xs[l]; };
-    for_rows2<KM>(a.L, lo, hi, [&](int i, const int (&q)[KM]) { ts[i] = shifted_row<T, KM>(a.L, gs, i, q, c, xv); });
+    for_rows<F16, KM>(a, lo, hi, [&](int i, const int (&q)[KM], int deg) {
+      ts[i] = shifted_row<T, F16, KM>(a, gs, i, q, deg, c, xs[i], xv);
+    });
   }
   if (a.side == 1) xt_partial<T>(a, lo, hi, xs, a.ypart + (size_t)blockIdx.x * a.m);
-  if (!grid_sync(a)) goto done;
+  if (!grid_bar_sync(bar)) goto done;
   if (a.side == 1) {
     reduce_y_global(a);
-    if (!grid_sync(a)) goto done;
+    if (!grid_bar_sync(bar)) goto done;
     load_y(a, ys);
   }
   // ---- r0 = b - A_hat x0; partial rho, |r|^2, |b|^2
   {
     auto tv = [&](int l) { return ts[l]; };
-    Acc<T> a_rho, a_rr, a_bb;
-    for_rows2<KM>(a.L, lo, hi, [&](int i, const int (&q)[KM]) {
+    Acc<T> acc[3];
+    for_rows<F16, KM>(a, lo, hi, [&](int i, const int (&q)[KM], int deg) {
       const T xi = xs[i];
       const T bi = (T)a.b[i];
-      const T ri = bi - (lam * (shifted_row<T, KM>(a.L, gs, i, q, c, tv) + e * xi) + data_row<T>(a, om, ys, i, xi));
+      const T ri = bi - (lam * (shifted_row<T, F16, KM>(a, gs, i, q, deg, c, ts[i], tv) + e * xi) + data_row<T>(a, om, ys, i, xi));
+      const T zi = dv[i] * ri;
       rs[i] = ri;
-      a_rho.add(ri, dv[i] * ri);
-      a_rr.add(ri, ri);
-      a_bb.add(bi, bi);
+      zs[i] = zi;
+      acc[0].add(ri, zi);
+      acc[1].add(ri, ri);
+      acc[2].add(bi, bi);
     });
-    double v[3] = {a_rho.get(), a_rr.get(), a_bb.get()};
-    block_reduce<3>(v, red);
+    block_reduce(acc, red);
     if (threadIdx.x == 0) {
       double* pb = a.part + (size_t)blockIdx.x * kParts;
       pb[1] = red[0];
@@ -343,10 +398,14 @@ __global__ void __launch_bounds__(kGThreads) pcg_grid_kernel(const GridPcg a) {
       pb[3] = red[2];
     }
   }
-  if (!grid_sync(a)) goto done;
-  rho = sum_parts(a.part, a.nb, kParts, 1);
-  rr = sum_parts(a.part, a.nb, kParts, 2);
-  bb = sum_parts(a.part, a.nb, kParts, 3);
+  if (!grid_bar_sync(bar)) goto done;
+  {
+    double v[3];
+    sum_parts<3>(a.part, a.nb, 1, v);
+    rho = v[0];
+    rr = v[1];
+    bb = v[2];
+  }
   if (bb > 0.0) {
     const double tol2 = a.tol * a.tol * bb;
     double rho_prev = 1.0;
@@ -363,41 +422,40 @@ __global__ void __launch_bounds__(kGThreads) pcg_grid_kernel(const GridPcg a) {
       {
         const bool first = it == 0;
         const T beta = (T)(first ? 0.0 : rho / rho_prev);
-        auto pn = [&](int l) -> T {
-          const T z = dv[l] * rs[l];
-          return first ? z : fma(beta, pold[l], z);
-        };
-        for_rows2<KM>(a.L, lo, hi, [&](int i, const int (&q)[KM]) {
-          ts[i] = shifted_row<T, KM>(a.L, gs, i, q, c, pn);
-          pnew[i] = pn(i);
+        auto pn = [&](int l) -> T { return first ? zs[l] : fma(beta, pold[l], zs[l]); };
+        for_rows<F16, KM>(a, lo, hi, [&](int i, const int (&q)[KM], int deg) {
+          const T pi = pn(i);
+          pnew[i] = pi;
+          ts[i] = shifted_row<T, F16, KM>(a, gs, i, q, deg, c, pi, pn);
         });
       }
       if (a.side == 1) {
         __syncthreads();
         xt_partial<T>(a, lo, hi, pnew, a.ypart + (size_t)blockIdx.x * a.m);
       }
-      if (!grid_sync(a)) goto done;
+      if (!grid_bar_sync(bar)) goto done;
       if (a.side == 1) {
         reduce_y_global(a);
-        if (!grid_sync(a)) goto done;
+        if (!grid_bar_sync(bar)) goto done;
         load_y(a, ys);
       }
       // ---- sweep A2b: q = lam ((L + cI) t + e p) + data(p); partial <p, q>
       {
         auto tv = [&](int l) { return ts[l]; };
-        Acc<T> a_pq;
-        for_rows2<KM>(a.L, lo, hi, [&](int i, const int (&q)[KM]) {
+        Acc<T> acc[1];
+        for_rows<F16, KM>(a, lo, hi, [&](int i, const int (&q)[KM], int deg) {
           const T pi = pnew[i];
-          const T qi = lam * (shifted_row<T, KM>(a.L, gs, i, q, c, tv) + e * pi) + data_row<T>(a, om, ys, i, pi);
+          const T qi = lam * (shifted_row<T, F16, KM>(a, gs, i, q, deg, c, ts[i], tv) + e * pi) + data_row<T>(a, om, ys, i, pi);
           qs[i] = qi;
-          a_pq.add(pi, qi);
+          acc[0].add(pi, qi);
         });
-        double v[1] = {a_pq.get()};
-        block_reduce<1>(v, red);
+        block_reduce(acc, red);
         if (threadIdx.x == 0) a.part[(size_t)blockIdx.x * kParts + 0] = red[0];
       }
-      if (!grid_sync(a)) goto done;
-      const double pq = sum_parts(a.part, a.nb, kParts, 0);
+      if (!grid_bar_sync(bar)) goto done;
+      double pqv[1];
+      sum_parts<1>(a.part, a.nb, 0, pqv);
+      const double pq = pqv[0];
       if (!(pq > 0.0)) {
         status = 2;
         break;
@@ -405,16 +463,30 @@ __global__ void __launch_bounds__(kGThreads) pcg_grid_kernel(const GridPcg a) {
       // ---- sweep B: x += alpha p, r -= alpha q; partial rho, |r|^2
       {
         const T alpha = (T)(rho / pq);
-        Acc<T> a_rho, a_rr;
-        for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-          xs[i] = fma(alpha, pnew[i], xs[i]);
-          const T ri = fma(-alpha, qs[i], rs[i]);
-          rs[i] = ri;
-          a_rho.add(ri, dv[i] * ri);
-          a_rr.add(ri, ri);
+        Acc<T> acc[2];
+        // chunk and vector starts are multiples of four rows
+        for (int i = lo + 4 * threadIdx.x; i < hi; i += 4 * blockDim.x) {
+          T xv[4], pv[4], rv[4], qv[4], dd4[4], zv[4];
+          ld4(xv, xs + i);
+          ld4(pv, pnew + i);
+          ld4(rv, rs + i);
+          ld4(qv, qs + i);
+          ld4(dd4, dv + i);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            xv[u] = fma(alpha, pv[u], xv[u]);
+            rv[u] = fma(-alpha, qv[u], rv[u]);
+            zv[u] = dd4[u] * rv[u];
+            if (i + u < hi) {
+              acc[0].add(rv[u], zv[u]);
+              acc[1].add(rv[u], rv[u]);
+            }
+          }
+          st4(xs + i, xv);
+          st4(rs + i, rv);
+          st4(zs + i, zv);
         }
-        double v[2] = {a_rho.get(), a_rr.get()};
-        block_reduce<2>(v, red);
+        block_reduce(acc, red);
         if (threadIdx.x == 0) {
           double* pb = a.part + (size_t)blockIdx.x * kParts;
           pb[1] = red[0];
@@ -422,10 +494,12 @@ __global__ void __launch_bounds__(kGThreads) pcg_grid_kernel(const GridPcg a) {
         }
       }
       ++it;
-      if (!grid_sync(a)) goto done;
+      if (!grid_bar_sync(bar)) goto done;
+      double v2[2];
+      sum_parts<2>(a.part, a.nb, 1, v2);
       rho_prev = rho;
-      rho = sum_parts(a.part, a.nb, kParts, 1);
-      rr = sum_parts(a.part, a.nb, kParts, 2);
+      rho = v2[0];
+      rr = v2[1];
     }
   }
   for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) a.x[i] = (double)xs[i];
@@ -445,29 +519,34 @@ done:
 
 namespace cr {
 
-// Largest block count that is co-resident for the kernel variant (float32 or
-// float64; 6 or up to kMaxSlots neighbour slots), at most two blocks of
-// kGThreads per SM (cooperative launch); 0 if it cannot run.
-const void* grid_kernel_fn(bool fp32, int K) {
-  const bool k6 = K <= 6;
-  return fp32 ? (k6 ? (const void*)pcg_grid_kernel<float, 6> : (const void*)pcg_grid_kernel<float, kMaxSlots>)
-              : (k6 ? (const void*)pcg_grid_kernel<double, 6> : (const void*)pcg_grid_kernel<double, kMaxSlots>);
+// Threads per block and largest block count that is co-resident for the kernel
+// variant (float32 or float64; neighbour table), at most one block of 1,024 or two
+// of 512 threads per SM (cooperative launch); 0 if it cannot run.
+static int grid_threads(const DevLap& L) { return L.nbr16 ? kGThreads16 : kGThreads; }
+const void* grid_kernel_fn(bool fp32, const DevLap& L) {
+  if (L.nbr16) return fp32 ? (const void*)pcg_grid_kernel<float, 6, true> : (const void*)pcg_grid_kernel<double, 6, true>;
+  const bool k6 = L.K <= 6;
+  return fp32 ? (k6 ? (const void*)pcg_grid_kernel<float, 6, false> : (const void*)pcg_grid_kernel<float, kMaxSlots, false>)
+              : (k6 ? (const void*)pcg_grid_kernel<double, 6, false>
+                    : (const void*)pcg_grid_kernel<double, kMaxSlots, false>);
 }
 
-int pcg_grid_blocks(bool fp32, int m, int K) {
+int pcg_grid_blocks(bool fp32, int m, const DevLap& L) {
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const size_t smem = sizeof(double) * (size_t)std::max(m, 1);
-  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, grid_kernel_fn(fp32, K), kGThreads, smem);
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, grid_kernel_fn(fp32, L), grid_threads(L), smem);
   if (e != cudaSuccess || per < 1) {
     cudaGetLastError();
     return 0;
   }
-  return sms * std::min(per, 2);
+  return sms * std::min(per, L.nbr16 ? 1 : 2);
 }
 
-size_t pcg_grid_work_elems(int n) { return (size_t)9 * n; }
+// vectors start at multiples of 16 rows, so that four rows load at once
+static size_t grid_stride(int n) { return ((size_t)n + 15) / 16 * 16; }
+size_t pcg_grid_work_elems(int n) { return 10 * grid_stride(n); }
 
 cudaError_t pcg_grid_launch(const PcgArgs& a, int side, const int* xc_ptr, const int* xc_row, const double* xc_val,
                             double* work, double* part, double* ypart, double* yglob, unsigned* bar, int* err,
@@ -493,15 +572,16 @@ cudaError_t pcg_grid_launch(const PcgArgs& a, int side, const int* xc_ptr, const
   g.omt64 = a.omt;
   const size_t word = a.fp32 ? sizeof(float) : sizeof(double);
   char* w = reinterpret_cast<char*>(work);
-  void** slots[9] = {&g.xs, &g.rs, &g.p0, &g.p1, &g.qs, &g.ts, &g.ds, &g.os, &g.gs};
-  for (int k = 0; k < 9; ++k) *slots[k] = w + (size_t)k * n * word;
+  void** slots[10] = {&g.xs, &g.rs, &g.p0, &g.p1, &g.qs, &g.ts, &g.ds, &g.os, &g.gs, &g.zs};
+  for (int k = 0; k < 10; ++k) *slots[k] = w + (size_t)k * grid_stride(n) * word;
+  g.idx = a.L.nbr16;
   g.part = part;
   g.ypart = ypart;
   g.yglob = yglob;
   g.bar = bar;
   g.err = err;
   g.nb = nb;
-  g.chunk = (n + nb - 1) / nb;
+  g.chunk = ((n + nb - 1) / nb + 3) / 4 * 4;
   g.tol = a.tol;
   g.maxit = a.maxit;
   g.stat = a.stat;
@@ -511,7 +591,7 @@ cudaError_t pcg_grid_launch(const PcgArgs& a, int side, const int* xc_ptr, const
   void* args[] = {&g};
   const size_t smem = sizeof(double) * (size_t)std::max(a.m, 1);
   count_launch();
-  return cudaLaunchCooperativeKernel(grid_kernel_fn(a.fp32 != 0, a.L.K), dim3(nb), dim3(kGThreads), args, smem, st);
+  return cudaLaunchCooperativeKernel(grid_kernel_fn(a.fp32 != 0, a.L), dim3(nb), dim3(grid_threads(a.L)), args, smem, st);
 }
 
 }  // namespace cr
