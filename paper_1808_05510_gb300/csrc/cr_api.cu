@@ -236,6 +236,11 @@ struct cr_problem {
   double *post_Ur = nullptr, *post_Zr = nullptr, *post_Vr = nullptr, *post_Pr = nullptr;
   double *post_small = nullptr, *post_Uh = nullptr, *post_Vh = nullptr;
   int post_ref_cap = 0;
+  // digit planes and row scales of P, V and the reference's factors (tensor-core pass)
+  uint16_t* post_dig[4] = {nullptr, nullptr, nullptr, nullptr};
+  double* post_scale[4] = {nullptr, nullptr, nullptr, nullptr};
+  int post_dig_cap[4] = {0, 0, 0, 0};
+  int* post_odd = nullptr;
   int64_t post_part_cap = 0, post_W_cols = 0;
   int64_t fcg_fallbacks = 0, learned_solves = 0, mixed_handovers = 0;
   // grid-wide PCG (grids the register-resident kernel does not take, or pcg_kernel = 2): work buffers
@@ -2985,6 +2990,11 @@ cr_status cr_svd_factors(cr_problem* p, double* Uh, int64_t ldu, double* sigma, 
   return sync(p);
 }
 
+// The solution pass runs on the tensor cores from this combined rank on, or from this many entries
+// (900^2: rank 16 0.13 against 0.11 ms, 24 0.135 against 0.137; 7,530^2: 1.6 against 2.6 ms at rank 1).
+constexpr int kPostTcRank = 24;
+constexpr int64_t kPostTcEntries = 1 << 22;
+
 cr_status cr_solution_report(cr_problem* p, int32_t nonneg, int32_t jr, const double* Ur, int64_t ldur,
                              const double* Zr, int64_t ldzr, const double* Vr, int64_t ldvr, double* W, int64_t ldw,
                              cr_solution_stats* out) {
@@ -3034,8 +3044,30 @@ cr_status cr_solution_report(cr_problem* p, int32_t nonneg, int32_t jr, const do
       p->post_W_cols = cw;
     }
   }
+  // tensor-core form: digits of the four factors, and the float64 pass behind it for
+  // factors that they cannot hold
+  const bool tc = j > 0 && (j + jr >= kPostTcRank || out->entries >= kPostTcEntries) && post_tc_blocks() > 0;
+  if (tc) {
+    if (!p->post_odd) TRY(dalloc(p, &p->post_odd, 1));
+    CUCHK(p, cudaMemsetAsync(p->post_odd, 0, sizeof(int), st));
+    const double* src[4] = {p->post_P, p->VV, p->post_Pr, p->post_Vr};
+    const int64_t lds[4] = {ny, 3 * (int64_t)nx, ny, nx};
+    for (int k = 0; k < 4; ++k) {
+      const int n = k % 2 == 0 ? ny : nx, r = k < 2 ? j : jr, cap = k < 2 ? p->rcap : p->post_ref_cap;
+      if (r == 0) continue;
+      if (r > p->post_dig_cap[k]) {
+        TRY(dalloc(p, &p->post_dig[k], post_tc_digit_elems(n, cap)));
+        if (!p->post_scale[k]) TRY(dalloc(p, &p->post_scale[k], (size_t)n));
+        p->post_dig_cap[k] = cap;
+      }
+      post_tc_digits(n, r, src[k], lds[k], p->post_dig[k], p->post_scale[k], p->post_odd, st);
+    }
+  }
   int64_t nparts = 0;
-  for (int64_t c0 = 0; c0 < nx; c0 += cw) nparts += post_tiles_parts(ny, (int)std::min<int64_t>(cw, nx - c0));
+  for (int64_t c0 = 0; c0 < nx; c0 += cw) {
+    const int ncols = (int)std::min<int64_t>(cw, nx - c0);
+    nparts += post_tiles_parts(ny, ncols) + (tc ? post_tc_parts(ny, ncols) : 0);
+  }
   if (nparts > p->post_part_cap) {
     TRY(dalloc(p, &p->post_part, (size_t)nparts * PS_N));
     p->post_part_cap = nparts;
@@ -3044,7 +3076,13 @@ cr_status cr_solution_report(cr_problem* p, int32_t nonneg, int32_t jr, const do
   int64_t off = 0;
   for (int64_t c0 = 0; c0 < nx; c0 += cw) {
     const int ncols = (int)std::min<int64_t>(cw, nx - c0);
-    post_tiles(ny, j, p->post_P, ny, p->VV, 3 * (int64_t)nx, jr, p->post_Pr, ny, p->post_Vr, nx, nonneg ? 1 : 0,
+    if (tc) {
+      post_tc_tiles(p->post_odd, ny, nx, j, p->post_dig[0], p->post_scale[0], p->post_dig[1], p->post_scale[1], jr,
+                    p->post_dig[2], p->post_scale[2], p->post_dig[3], p->post_scale[3], nonneg ? 1 : 0, (int)c0, ncols,
+                    W ? p->post_W : nullptr, ny, p->post_part + off * PS_N, st);
+      off += post_tc_parts(ny, ncols);
+    }
+    post_tiles(tc ? p->post_odd : nullptr, ny, j, p->post_P, ny, p->VV, 3 * (int64_t)nx, jr, p->post_Pr, ny, p->post_Vr, nx, nonneg ? 1 : 0,
                (int)c0, ncols, W ? p->post_W : nullptr, ny, p->post_part + off * PS_N, st);
     off += post_tiles_parts(ny, ncols);
     if (W) {

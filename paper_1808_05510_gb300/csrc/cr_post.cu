@@ -1,4 +1,5 @@
-// Post-processing of a greedy solution W = U Z V^T: one tiled float64 pass
+// Post-processing of a greedy solution W = U Z V^T: one tiled float64 pass (the
+// form for small ranks and for factors that cr_post_tc.cu cannot scale)
 // that forms W on chip (64 x 64 tiles, never the whole ny x nx matrix),
 // optionally projects it onto the nonnegative orthant (Sec. 4, dropping the
 // nonnegativity constraint), compares it with a reference W* = U* Z* V*^T
@@ -10,6 +11,7 @@
 #include <algorithm>
 
 #include "cr_common.cuh"
+#include "cr_post_stats.cuh"
 
 namespace cr {
 
@@ -18,38 +20,6 @@ namespace {
 constexpr int PT = 64;   // output tile edge
 constexpr int PK = 16;   // reduction step staged in shared memory
 constexpr int PTHREADS = 256;
-
-__device__ __forceinline__ double stat_op(int q, double a, double b) {
-  if (q == PS_MIN) return fmin(a, b);
-  if (q == PS_MAX || q == PS_MAXABS) return fmax(a, b);
-  return a + b;
-}
-
-__device__ __forceinline__ double stat_identity(int q) {
-  if (q == PS_MIN) return INFINITY;
-  if (q == PS_MAX) return -INFINITY;
-  return 0.0;
-}
-
-// fixed-order block combination of per-thread statistics; thread 0 writes out[0..PS_N)
-__device__ void block_stats(double (&v)[PS_N], double* out) {
-  __shared__ double scr[PTHREADS / 32][PS_N];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int q = 0; q < PS_N; ++q)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[q] = stat_op(q, v[q], __shfl_down_sync(0xffffffffu, v[q], o));
-  if (lane == 0)
-#pragma unroll
-    for (int q = 0; q < PS_N; ++q) scr[wid][q] = v[q];
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int q = 0; q < PS_N; ++q) {
-      double a = scr[0][q];
-      for (int w = 1; w < nw; ++w) a = stat_op(q, a, scr[w][q]);
-      out[q] = a;
-    }
-}
 
 // acc[a][b] += sum_k P(i0 + tx + 16a, k) V(c0 + ty + 16b, k), k < K; P col-major (ld ldp),
 // V(c, k) at V[c + k * ldv].  Rows or columns past the matrix read as zero.
@@ -88,7 +58,8 @@ __device__ __forceinline__ void tile_product(int nrow, int ncol, int K, const do
 // Tile t (row-tile fastest) belongs to CTA t mod gridDim.x.  out (may be null)
 // receives P(W) for the columns of this launch, column c at out + (c - col0) * ldo.
 // part[blockIdx.x * PS_N + q] receives the CTA's statistics.
-__global__ void __launch_bounds__(PTHREADS) post_tile_kernel(int ny, int j, const double* __restrict__ P,
+// run_if (may be null): the pass runs only where *run_if is set, else it leaves empty statistics.
+__global__ void __launch_bounds__(PTHREADS) post_tile_kernel(const int* __restrict__ run_if, int ny, int j, const double* __restrict__ P,
                                                              int64_t ldp, const double* __restrict__ V, int64_t ldv,
                                                              int jr, const double* __restrict__ Pr, int64_t ldpr,
                                                              const double* __restrict__ Vr, int64_t ldvr, int nonneg,
@@ -103,7 +74,8 @@ __global__ void __launch_bounds__(PTHREADS) post_tile_kernel(int ny, int j, cons
   double s[PS_N];
 #pragma unroll
   for (int q = 0; q < PS_N; ++q) s[q] = stat_identity(q);
-  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+  const int64_t nrun = run_if && !*run_if ? 0 : ntiles;
+  for (int64_t t = blockIdx.x; t < nrun; t += gridDim.x) {
     const int i0 = (int)(t % rt) * PT, c0 = col0 + (int)(t / rt) * PT;
     double acc[4][4], accr[4][4];
 #pragma unroll
@@ -120,23 +92,12 @@ __global__ void __launch_bounds__(PTHREADS) post_tile_kernel(int ny, int j, cons
         const int i = i0 + tx + 16 * a;
         if (i >= ny || c >= cend) continue;
         const double w = acc[a][b], wr = accr[a][b];
-        if (w < 0.0) {
-          s[PS_NNEG] += 1.0;
-          s[PS_NEG2] = fma(w, w, s[PS_NEG2]);
-        }
-        s[PS_MIN] = fmin(s[PS_MIN], w);
-        s[PS_MAX] = fmax(s[PS_MAX], w);
-        s[PS_W2] = fma(w, w, s[PS_W2]);
-        const double pw = (nonneg && w < 0.0) ? 0.0 : w;
-        const double d = pw - wr;
-        s[PS_REF2] = fma(wr, wr, s[PS_REF2]);
-        s[PS_DIFF2] = fma(d, d, s[PS_DIFF2]);
-        s[PS_MAXABS] = fmax(s[PS_MAXABS], fabs(d));
+        const double pw = stat_add(s, w, wr, nonneg);
         if (out) out[(int64_t)i + (int64_t)(c - col0) * ldo] = pw;
       }
     }
   }
-  block_stats(s, part + (int64_t)blockIdx.x * PS_N);
+  block_stats<PTHREADS>(s, part + (int64_t)blockIdx.x * PS_N);
 }
 
 // out[q] = the combination of part[p * PS_N + q] over p < nparts, in a fixed order
@@ -147,7 +108,7 @@ __global__ void post_reduce_kernel(int nparts, const double* __restrict__ part, 
   for (int p = threadIdx.x; p < nparts; p += blockDim.x)
 #pragma unroll
     for (int q = 0; q < PS_N; ++q) s[q] = stat_op(q, s[q], part[(int64_t)p * PS_N + q]);
-  block_stats(s, out);
+  block_stats<PTHREADS>(s, out);
 }
 
 }  // namespace
@@ -169,12 +130,12 @@ int post_tiles_parts(int ny, int ncols) {
   return (int)std::min<int64_t>(post_blocks(), std::max<int64_t>(ntiles, 1));
 }
 
-void post_tiles(int ny, int j, const double* P, int64_t ldp, const double* V, int64_t ldv, int jr,
+void post_tiles(const int* run_if, int ny, int j, const double* P, int64_t ldp, const double* V, int64_t ldv, int jr,
                 const double* Pr, int64_t ldpr, const double* Vr, int64_t ldvr, int nonneg, int col0, int ncols,
                 double* out, int64_t ldo, double* part, cudaStream_t st) {
   const int nb = post_tiles_parts(ny, ncols);
   count_launch();
-  post_tile_kernel<<<nb, PTHREADS, 0, st>>>(ny, j, P, ldp, V, ldv, jr, Pr, ldpr, Vr, ldvr, nonneg, col0, ncols,
+  post_tile_kernel<<<nb, PTHREADS, 0, st>>>(run_if, ny, j, P, ldp, V, ldv, jr, Pr, ldpr, Vr, ldvr, nonneg, col0, ncols,
                                             out, ldo, part);
 }
 
