@@ -53,7 +53,7 @@ constexpr int kMaxRefine = 8;
 const char* const kBarrierTimeout = "grid-wide PCG barrier timed out";
 
 enum {
-  DS_UN2 = 0, DS_VN2 = 1, DS_NB = 2, DS_NA = 3, DS_DW = 4, /*5*/ DS_ZKZ = 6, DS_ZF = 7, DS_RN = 8, DS_V0 = 9,
+  DS_UN2 = 0, DS_VN2 = 1, DS_NB = 2, DS_NA = 3, DS_DW = 4, /*5*/ DS_ZKZ = 6, DS_ZF = 7, DS_RN = 8, DS_V0 = 9, DS_NNEW = 10,
   DS_GS = 16, DS_FCG = 24, DS_REF = 30, DS_COUNT = 32
 };
 
@@ -266,6 +266,7 @@ struct cr_problem {
   double *QL = nullptr, *CL = nullptr, *QR = nullptr, *CRm = nullptr, *Cx = nullptr, *Cx2 = nullptr, *Ep = nullptr,
          *CE = nullptr, *CP = nullptr, *T1 = nullptr, *T2 = nullptr, *gram = nullptr, *tmat = nullptr;
   int nQL = 0, nQR = 0, nQX = 0;
+  double* bcoef = nullptr;   // coefficients of the columns being appended, both grids
   std::vector<int> qr_step;  // greedy step that created right-basis vector nQX + i
   int64_t ldcl = 0, ldcr = 0, ldcx = 0, ldcp = 0, ldm = 0;
   double* ws = nullptr;
@@ -1485,34 +1486,51 @@ void refresh_E(cr_problem* p) {
   mask_residual(p->ny, m, p->OmY, p->Om, p->ny, p->E, st);
 }
 
-// Append UU/VV columns 3q..3q+2 to the residual-norm bases.
+// Append UU/VV columns 3q..3q+2 to the residual-norm bases (cr_basis.cu): block
+// Gram-Schmidt twice, then the coefficients of the new columns.
 cr_status grow_bases(cr_problem* p, int q) {
   cudaStream_t st = p->st;
-  for (int s = 0; s < 3; ++s) {
-    const double* col = p->UU + (size_t)(3 * q + s) * p->ny;
-    double* dst = p->QL + (size_t)p->nQL * p->ny;
-    copy(p->ny, col, dst, st);
-    double ratio = 0.0;
-    TRY(cgs2(p, p->ny, p->QL, p->ny, p->nQL, dst, &ratio));
-    if (ratio > 1e-12) ++p->nQL;
+  PanelArgs a;
+  a.n[0] = p->ny;
+  a.n[1] = p->nx;
+  a.k[0] = p->nQL;
+  a.k[1] = p->nQR;
+  a.A[0] = p->QL;
+  a.A[1] = p->QR;
+  a.src[0] = p->UU + (size_t)3 * q * p->ny;
+  a.src[1] = p->VV + (size_t)3 * q * p->nx;
+  a.w[0] = p->QL + (size_t)p->nQL * p->ny;
+  a.w[1] = p->QR + (size_t)p->nQR * p->nx;
+  const int64_t ldc = p->m + 3 * (int64_t)p->rcap;
+  for (int g = 0; g < 2; ++g) {
+    a.lda[g] = a.ldw[g] = a.lds[g] = a.n[g];
+    a.out[g] = p->bcoef + (size_t)g * 3 * ldc;
+    a.ldo[g] = ldc;
+    a.count[g] = p->ds + DS_NNEW + g;
   }
-  for (int s = 0; s < 3; ++s)
-    gemv_t(p->ny, p->nQL, p->QL, p->ny, p->UU + (size_t)(3 * q + s) * p->ny, p->CL + (size_t)(3 * q + s) * p->ldcl,
-           1, 1.0, 0.0, st);
-  for (int s = 0; s < 3; ++s) {
-    const double* col = p->VV + (size_t)(3 * q + s) * p->nx;
-    double* dst = p->QR + (size_t)p->nQR * p->nx;
-    copy(p->nx, col, dst, st);
-    double ratio = 0.0;
-    TRY(cgs2(p, p->nx, p->QR, p->nx, p->nQR, dst, &ratio));
-    if (ratio > 1e-12) {
-      ++p->nQR;
-      p->qr_step.push_back(q);
-    }
+  panel_copy(a, st);
+  for (int pass = 0; pass < 2; ++pass) {
+    panel_t(a, 3, st);
+    panel_n(a, st);
+    panel_orth(a, pass == 0, st);
   }
-  for (int s = 0; s < 3; ++s)
-    gemv_t(p->nx, p->nQR, p->QR, p->nx, p->VV + (size_t)(3 * q + s) * p->nx,
-           p->CRm + (size_t)(p->m + 3 * q + s) * p->ldcr, 1, 1.0, 0.0, st);
+  // coefficients of the three columns in the grown bases (a dropped column left zeros)
+  PanelArgs c = a;
+  for (int g = 0; g < 2; ++g) {
+    c.k[g] = a.k[g] + 3;
+    c.w[g] = a.src[g];
+    c.ldw[g] = a.lds[g];
+  }
+  c.out[0] = p->CL + (size_t)3 * q * p->ldcl;
+  c.ldo[0] = p->ldcl;
+  c.out[1] = p->CRm + (size_t)(p->m + 3 * q) * p->ldcr;
+  c.ldo[1] = p->ldcr;
+  panel_t(c, 3, st);
+  TRY(readback(p, DS_NNEW, 2, false));
+  p->nQL += (int)p->hs->ds[DS_NNEW];
+  const int nr = (int)p->hs->ds[DS_NNEW + 1];
+  p->nQR += nr;
+  for (int k = 0; k < nr; ++k) p->qr_step.push_back(q);
   return CR_OK;
 }
 
@@ -1530,14 +1548,28 @@ cr_status grow_projections(cr_problem* p, int q) {
   lap_apply(p->Lx, vq, vq + nx, 0.0, st);
   lap_apply(p->Lx, vq + nx, vq + 2 * nx, 0.0, st);
   const int64_t ldu = 3 * (int64_t)ny, ldv = 3 * (int64_t)nx;
-  gemv_t(ny, q + 1, p->UU, ldu, uq + ny, p->A1 + q * ld, 1, 1.0, 0.0, st);
-  gemv_t(ny, q + 1, p->UU, ldu, uq + 2 * ny, p->A2 + q * ld, 1, 1.0, 0.0, st);
-  gemv_t(nx, q + 1, p->VV, ldv, vq + nx, p->B1 + q * ld, 1, 1.0, 0.0, st);
-  gemv_t(nx, q + 1, p->VV, ldv, vq + 2 * nx, p->B2 + q * ld, 1, 1.0, 0.0, st);
-  mirror_col(q, p->A1, ld, 1, 0, st);
-  mirror_col(q, p->A2, ld, 1, 0, st);
-  mirror_col(q, p->B1, ld, 1, 0, st);
-  mirror_col(q, p->B2, ld, 1, 0, st);
+  PanelArgs b;  // column and row q of A1, A2 (y grid) and B1, B2 (x grid)
+  b.n[0] = ny;
+  b.n[1] = nx;
+  b.k[0] = b.k[1] = q + 1;
+  b.A[0] = p->UU;
+  b.A[1] = p->VV;
+  b.lda[0] = ldu;
+  b.lda[1] = ldv;
+  b.w[0] = uq + ny;
+  b.w[1] = vq + nx;
+  b.ldw[0] = ny;
+  b.ldw[1] = nx;
+  double* const m1[2] = {p->A1, p->B1};
+  double* const m2[2] = {p->A2, p->B2};
+  for (int g = 0; g < 2; ++g) {
+    b.out[g] = m1[g] + q * ld;
+    b.out2[g] = m2[g] + q * ld;
+    b.row[g][0] = m1[g] + q;
+    b.row[g][1] = m2[g] + q;
+  }
+  b.ldrow = ld;
+  panel_t(b, 2, st);
   spmv_xt(m, p->xc_ptr, p->xc_row, p->xc_val, vq, p->H + q, ld, st);
   gemv_t(ny, m, p->OmY, ny, uq, p->P + q, ld, 1.0, 0.0, st);
   omega_times(ny, m, p->Om, ny, uq, p->Bnm, st);
@@ -1589,26 +1621,16 @@ cr_status eig_sync(cr_problem* p) {
   prof_begin(p, CR_PHASE_BASIS);
   while (p->eq < j) {
     const int q = p->eq, n1 = q + 1;
-    fill(1, 1.0, p->eQa + q + q * ld, st);   // blockdiag(Qa, 1): the rest of row and column q is zero
-    fill(1, 1.0, p->eQb + q + q * ld, st);
     double* za = p->ebord;
     double* zb = p->ebord + ld + 1;
-    if (q > 0) {
-      gemv_t(q, q, p->eQa, ld, p->A1 + q * ld, za, 1, 1.0, 0.0, st);
-      gemv_t(q, q, p->eQb, ld, p->B1 + q * ld, zb, 1, 1.0, 0.0, st);
-    }
-    copy(1, p->A1 + q + q * ld, za + q, st);
-    copy(1, p->B1 + q + q * ld, zb + q, st);
+    basis_border(q, ld, p->eQa, p->eQb, p->A1, p->B1, za, zb, st);  // blockdiag(Q, 1): the rest of row and column q is zero
     const double* d[2] = {p->ela, p->elb};
     const double* z[2] = {za, zb};
     const double* al[2] = {za + q, zb + q};
     double* mu[2] = {p->ela, p->elb};
     double* W[2] = {p->eW, p->eW + (size_t)n1 * n1};
     CUCHK(p, arrow_update(q, (int)ld, d, z, al, mu, W, p->earw, st));
-    gemm(n1, n1, n1, 1.0, MatView{p->eQa, 1, ld}, MatView{W[0], 1, n1}, 0.0, p->eQa2, 1, ld, p->ws, p->ws_elems,
-         st);
-    gemm(n1, n1, n1, 1.0, MatView{p->eQb, 1, ld}, MatView{W[1], 1, n1}, 0.0, p->eQb2, 1, ld, p->ws, p->ws_elems,
-         st);
+    basis_product(n1, ld, p->eQa, p->eQb, W[0], W[1], p->eQa2, p->eQb2, st);
     std::swap(p->eQa, p->eQa2);
     std::swap(p->eQb, p->eQb2);
     ++p->eq;
@@ -2463,6 +2485,7 @@ cr_status cr_create(const cr_problem_desc* d_in, const cr_options* o, cr_problem
   p->ldcx = 3 * (int64_t)rc;
   p->ldcp = 3 * (int64_t)rc + m;
   p->ldm = m + 3 * (int64_t)rc;
+  CK(dalloc(p, &p->bcoef, (size_t)6 * (3 * rc + m)));
   CK(dalloc(p, &p->QL, (size_t)ny * (3 * rc + m)));
   CK(dalloc(p, &p->CL, (size_t)p->ldcl * 3 * rc));
   CK(dalloc(p, &p->QR, (size_t)nx * (3 * rc + m)));

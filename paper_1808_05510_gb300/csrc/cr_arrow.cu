@@ -199,19 +199,23 @@ __global__ void arrow_roots_kernel(ArrowArgs a) {
 }
 
 // Loewner couplings: zh_t^2 = -prod_r (root_r - d_t) / prod_{s != t} (d_s - d_t).
+// One warp per pole: each lane multiplies every 32nd ratio (ratios of neighbouring
+// root and pole stay near 1), then the lanes' products in a fixed tree.  One thread
+// per pole made it a chain of k float64 divisions: 71 us at k = 120.
 __global__ void arrow_zhat_kernel(ArrowArgs a) {
   const int s = blockIdx.y;
   ArrowWork w = work_of(a.work + s * a.side_stride, a.nmax);
   const int k = w.meta[0];
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (t >= k || w.meta[3]) return;
   const double dt = w.dl[t];
-  double p = w.root[k] - dt;
-  for (int r = 0; r < k; ++r) {
-    p *= (w.root[r] - dt);
-    if (r != t) p /= (w.dl[r] - dt);
+  double p = lane == 0 ? w.root[k] - dt : 1.0;
+  for (int r = lane; r < k; r += 32) {
+    const double num = w.root[r] - dt;
+    p *= r != t ? num / (w.dl[r] - dt) : num;
   }
-  w.zh[t] = copysign(sqrt(fabs(p)), w.zl[t]);
+  for (int o = 16; o > 0; o >>= 1) p *= __shfl_xor_sync(0xffffffffu, p, o);
+  if (lane == 0) w.zh[t] = copysign(sqrt(fabs(p)), w.zl[t]);
 }
 
 // Eigenvectors, one warp per eigenpair: deflated pairs (d_i, e_i) and the k + 1
@@ -316,11 +320,14 @@ cudaError_t arrow_update(int n, int nmax, const double* const d[2], const double
   count_launch();
   arrow_prep_kernel<<<dim3(1, 2), 256, smem, st>>>(a);
   const int wpb = 8;  // warps per block
+  // a root takes tens of float64 divisions a lane, which share one pipe per SM: two warps a block
+  // spread the roots over all SMs (240 roots a side: eight warps a block 263 us)
+  const int wpr = 2;
   count_launch();
-  arrow_roots_kernel<<<dim3((n + 1 + wpb - 1) / wpb, 2), 32 * wpb, 0, st>>>(a);
+  arrow_roots_kernel<<<dim3((n + 1 + wpr - 1) / wpr, 2), 32 * wpr, 0, st>>>(a);
   if (n > 0) {
     count_launch();
-    arrow_zhat_kernel<<<dim3((n + 127) / 128, 2), 128, 0, st>>>(a);
+    arrow_zhat_kernel<<<dim3((n + wpr - 1) / wpr, 2), 32 * wpr, 0, st>>>(a);
   }
   count_launch();
   arrow_vectors_kernel<<<dim3((n + 1 + wpb - 1) / wpb, 2), 32 * wpb, 0, st>>>(a);

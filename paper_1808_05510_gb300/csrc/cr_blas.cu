@@ -36,19 +36,25 @@ __global__ void gemm_kernel(int M, int N, int K, MatView A, MatView B, int kchun
   const int k0 = s * kchunk, k1 = min(K, k0 + kchunk);
   const bool a_unit_i = A.si == 1;
   const bool b_unit_k = B.si == 1;  // B(k, l): k is B's "i" index
-  double acc = 0.0;
+  // this thread's element of the two panels at column kk; the next ones are loaded while the
+  // current ones are multiplied
+  const int iq = a_unit_i ? tx : ty, ka = a_unit_i ? ty : tx;
+  const int kb = b_unit_k ? tx : ty, lq = b_unit_k ? ty : tx;
+  auto la = [&](int kk) {
+    const int i = i0 + iq, k = kk + ka;
+    return (i < M && k < k1) ? A.ptr[(int64_t)i * A.si + (int64_t)k * A.sk] : 0.0;
+  };
+  auto lb = [&](int kk) {
+    const int k = kk + kb, l = l0 + lq;
+    return (k < k1 && l < N) ? B.ptr[(int64_t)k * B.si + (int64_t)l * B.sk] : 0.0;
+  };
+  double acc = 0.0, ra = la(k0), rb = lb(k0);
   for (int kk = k0; kk < k1; kk += TB) {
-    {
-      const int iq = a_unit_i ? tx : ty, kq = a_unit_i ? ty : tx;
-      const int i = i0 + iq, k = kk + kq;
-      As[kq][iq] = (i < M && k < k1) ? A.ptr[(int64_t)i * A.si + (int64_t)k * A.sk] : 0.0;
-    }
-    {
-      const int kq = b_unit_k ? tx : ty, lq = b_unit_k ? ty : tx;
-      const int k = kk + kq, l = l0 + lq;
-      Bs[kq][lq] = (k < k1 && l < N) ? B.ptr[(int64_t)k * B.si + (int64_t)l * B.sk] : 0.0;
-    }
+    As[ka][iq] = ra;
+    Bs[kb][lq] = rb;
     __syncthreads();
+    ra = la(kk + TB);
+    rb = lb(kk + TB);
 #pragma unroll
     for (int q = 0; q < TB; ++q) acc = fma(As[q][ty], Bs[q][tx], acc);
     __syncthreads();

@@ -419,6 +419,40 @@ cudaError_t galerkin_assemble_tc(int n, int j, int m, const void* hi, const void
 }  // namespace cr
 
 namespace cr {
+// ---------------------------------------------------------------- cr_basis.cu
+// Panel operations on both grids (0: y, 1: x) in one launch: A is n x k with
+// leading dimension lda, w up to three columns with leading dimension ldw.
+struct PanelArgs {
+  int n[2] = {0, 0}, k[2] = {0, 0};
+  const double* A[2] = {nullptr, nullptr};
+  int64_t lda[2] = {0, 0};
+  const double* w[2] = {nullptr, nullptr};  // written by panel_n, panel_copy, panel_orth
+  int64_t ldw[2] = {0, 0};
+  double* out[2] = {nullptr, nullptr};      // coefficients, column s at out + s ldo
+  int64_t ldo[2] = {0, 0};
+  double* out2[2] = {nullptr, nullptr};     // place of column 1 if not out + ldo
+  double* row[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // mirrored copies (columns 0, 1), stride ldrow
+  int64_t ldrow = 0;
+  const double* src[2] = {nullptr, nullptr};  // the three source columns, leading dimension lds
+  int64_t lds[2] = {0, 0};
+  double* count[2] = {nullptr, nullptr};
+};
+// out(p, s) = A(:, p)^T w_s for nv = 2 or 3 columns
+void panel_t(const PanelArgs& a, int nv, cudaStream_t st);
+// w_s -= A out(:, s), three columns
+void panel_n(const PanelArgs& a, cudaStream_t st);
+// w_s = src_s, three columns
+void panel_copy(const PanelArgs& a, cudaStream_t st);
+// Orthonormalise the three columns w; first: drop those whose norm fell to 1e-12 of the source's
+// (accepted ones to the front, zeros behind, *count = their number)
+void panel_orth(const PanelArgs& a, bool first, cudaStream_t st);
+// z = Q^T (border column q of A1 / B1), z_q its diagonal entry, Q(q, q) = 1
+void basis_border(int q, int64_t ld, double* Qa, double* Qb, const double* A1, const double* B1, double* za, double* zb,
+                  cudaStream_t st);
+// O = Q W for both eigenbases (n1 x n1; W with leading dimension n1)
+void basis_product(int n1, int64_t ld, const double* Qa, const double* Qb, const double* Wa, const double* Wb, double* Oa,
+                   double* Ob, cudaStream_t st);
+
 // ---------------------------------------------------------------- cr_small.cu
 // g[3p+s] = coef_s * sum_q Zop(p, q) h[3q + 2 - s], coef = (lam, 2 lam, lam), Zop = Z or Z^T
 void zcoef(int j, const double* Z, int64_t ldz, int trans, const double* h, double lam, double* g, cudaStream_t st);
