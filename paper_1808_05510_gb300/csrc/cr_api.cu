@@ -188,6 +188,8 @@ struct cr_problem {
   DevXLocal xl;
   double* OmY = nullptr;
   uint8_t* Om = nullptr;
+  int *om_ptr = nullptr, *om_row = nullptr;  // per injection the shorter of its unobserved (om_full) and observed rows
+  uint8_t* om_full = nullptr;
   double *UU = nullptr, *VV = nullptr, *Z = nullptr, *Zprev = nullptr;
   double *A1 = nullptr, *A2 = nullptr, *B1 = nullptr, *B2 = nullptr, *H = nullptr, *P = nullptr, *G = nullptr,
          *F = nullptr, *E = nullptr, *Mzh = nullptr;
@@ -1510,7 +1512,7 @@ cr_status grow_bases(cr_problem* p, int q) {
   }
   panel_copy(a, st);
   for (int pass = 0; pass < 2; ++pass) {
-    panel_t(a, 3, st);
+    panel_t(a, st);
     panel_n(a, st);
     panel_orth(a, pass == 0, st);
   }
@@ -1525,7 +1527,7 @@ cr_status grow_bases(cr_problem* p, int q) {
   c.ldo[0] = p->ldcl;
   c.out[1] = p->CRm + (size_t)(p->m + 3 * q) * p->ldcr;
   c.ldo[1] = p->ldcr;
-  panel_t(c, 3, st);
+  panel_t(c, st);
   TRY(readback(p, DS_NNEW, 2, false));
   p->nQL += (int)p->hs->ds[DS_NNEW];
   const int nr = (int)p->hs->ds[DS_NNEW + 1];
@@ -1548,7 +1550,9 @@ cr_status grow_projections(cr_problem* p, int q) {
   lap_apply(p->Lx, vq, vq + nx, 0.0, st);
   lap_apply(p->Lx, vq + nx, vq + 2 * nx, 0.0, st);
   const int64_t ldu = 3 * (int64_t)ny, ldv = 3 * (int64_t)nx;
-  PanelArgs b;  // column and row q of A1, A2 (y grid) and B1, B2 (x grid)
+  // u_p^T [u, L u, L^2 u]_q: the second and third are column and row q of A1, A2 (y grid) and B1, B2
+  // (x grid), the first enters every G_a
+  PanelArgs b;
   b.n[0] = ny;
   b.n[1] = nx;
   b.k[0] = b.k[1] = q + 1;
@@ -1556,26 +1560,24 @@ cr_status grow_projections(cr_problem* p, int q) {
   b.A[1] = p->VV;
   b.lda[0] = ldu;
   b.lda[1] = ldv;
-  b.w[0] = uq + ny;
-  b.w[1] = vq + nx;
+  b.w[0] = uq;
+  b.w[1] = vq;
   b.ldw[0] = ny;
   b.ldw[1] = nx;
   double* const m1[2] = {p->A1, p->B1};
   double* const m2[2] = {p->A2, p->B2};
   for (int g = 0; g < 2; ++g) {
-    b.out[g] = m1[g] + q * ld;
-    b.out2[g] = m2[g] + q * ld;
-    b.row[g][0] = m1[g] + q;
-    b.row[g][1] = m2[g] + q;
+    b.at[g][0] = p->bcoef + (size_t)g * ld;
+    b.at[g][1] = m1[g] + q * ld;
+    b.at[g][2] = m2[g] + q * ld;
+    b.row[g][1] = m1[g] + q;
+    b.row[g][2] = m2[g] + q;
   }
   b.ldrow = ld;
-  panel_t(b, 2, st);
+  panel_t(b, st);
   spmv_xt(m, p->xc_ptr, p->xc_row, p->xc_val, vq, p->H + q, ld, st);
   gemv_t(ny, m, p->OmY, ny, uq, p->P + q, ld, 1.0, 0.0, st);
-  omega_times(ny, m, p->Om, ny, uq, p->Bnm, st);
-  gemm(q + 1, m, ny, 1.0, MatView{p->UU, ldu, 1}, MatView{p->Bnm, 1, ny}, 0.0, p->G + q * ld, 1, ld * ld, p->ws,
-       p->ws_elems, st);
-  mirror_col(q, p->G, ld, m, ld * ld, st);
+  omega_border(q, m, p->UU, ldu, p->bcoef, p->om_ptr, p->om_row, p->om_full, p->G, ld, st);
   return grow_bases(p, q);
 }
 
@@ -2409,6 +2411,21 @@ cr_status cr_create(const cr_problem_desc* d_in, const cr_options* o, cr_problem
     for (int64_t a = 0; a < m; ++a) on2 += g1[a + a * m];
     p->Dnorm = std::sqrt(std::max(dn2, 0.0));
     p->OmYn2 = on2;
+  }
+  {
+    std::vector<int> zp(m + 1, 0), zr;
+    std::vector<uint8_t> full(m, 0);
+    for (int64_t a = 0; a < m; ++a) {
+      int64_t ones = 0;
+      for (int64_t i = 0; i < ny; ++i) ones += om[i + a * ny];
+      full[a] = 2 * ones >= ny;
+      for (int64_t i = 0; i < ny; ++i)
+        if ((om[i + a * ny] != 0) != (full[a] != 0)) zr.push_back((int)i);
+      zp[a + 1] = (int)zr.size();
+    }
+    CK(upload(p, &p->om_ptr, zp));
+    CK(upload(p, &p->om_row, zr));
+    CK(upload(p, &p->om_full, full));
   }
   CK(upload(p, &p->OmY, omy));
   CK(upload(p, &p->Om, om));

@@ -430,15 +430,19 @@ struct PanelArgs {
   int64_t ldw[2] = {0, 0};
   double* out[2] = {nullptr, nullptr};      // coefficients, column s at out + s ldo
   int64_t ldo[2] = {0, 0};
-  double* out2[2] = {nullptr, nullptr};     // place of column 1 if not out + ldo
-  double* row[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // mirrored copies (columns 0, 1), stride ldrow
+  double* at[2][3] = {};                    // place of column s if not out + s ldo
+  double* row[2][3] = {};                   // mirrored copy of column s, stride ldrow
   int64_t ldrow = 0;
   const double* src[2] = {nullptr, nullptr};  // the three source columns, leading dimension lds
   int64_t lds[2] = {0, 0};
   double* count[2] = {nullptr, nullptr};
 };
-// out(p, s) = A(:, p)^T w_s for nv = 2 or 3 columns
-void panel_t(const PanelArgs& a, int nv, cudaStream_t st);
+// out(p, s) = A(:, p)^T w_s, three columns
+void panel_t(const PanelArgs& a, cudaStream_t st);
+// Column and row q of every G_a = U^T diag(Omega_a) U (u_p at UU + p ldu), from D(p) = u_p^T u_q and
+// row lists: the unobserved rows of injection a (full[a]) or its observed ones
+void omega_border(int q, int m, const double* UU, int64_t ldu, const double* D, const int* zp, const int* zrow,
+                  const uint8_t* full, double* G, int64_t ld, cudaStream_t st);
 // w_s -= A out(:, s), three columns
 void panel_n(const PanelArgs& a, cudaStream_t st);
 // w_s = src_s, three columns
@@ -456,14 +460,10 @@ void basis_product(int n1, int64_t ld, const double* Qa, const double* Qb, const
 // ---------------------------------------------------------------- cr_small.cu
 // g[3p+s] = coef_s * sum_q Zop(p, q) h[3q + 2 - s], coef = (lam, 2 lam, lam), Zop = Z or Z^T
 void zcoef(int j, const double* Z, int64_t ldz, int trans, const double* h, double lam, double* g, cudaStream_t st);
-// A(col, p) = A(p, col) for p < col, in `batch` matrices spaced `stride` apart
-void mirror_col(int col, double* A, int64_t ld, int batch, int64_t stride, cudaStream_t st);
 // Z(j, q) = Z(q, j) = 0 for q <= j
 void zero_border(int j, double* Z, int64_t ld, cudaStream_t st);
 // E = OmY - Om o E  (ny x m, ld ny)
 void mask_residual(int n, int m, const double* OmY, const uint8_t* Om, int64_t ldo, double* E, cudaStream_t st);
-// B(i, a) = Om(i, a) * u(i)
-void omega_times(int n, int m, const uint8_t* Om, int64_t ldo, const double* u, double* B, cudaStream_t st);
 // out[0] = sum_{i<r, l<c} A(i,l) B(i,l) (single deterministic reduction)
 void mat_dot(int r, int c, const double* A, int64_t lda, const double* B, int64_t ldb, double* out, cudaStream_t st);
 // out[0] = sum Om (P - Y)^2, out[1] = sum Om Y^2 over n x m (P, Y, Om contiguous, ld n)

@@ -49,13 +49,6 @@ __global__ void zcoef_kernel(int j, const double* __restrict__ Z, int64_t ldz, i
   g[t] = coef * acc;
 }
 
-__global__ void mirror_col_kernel(int col, double* A, int64_t ld, int64_t stride) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= col) return;
-  double* a = A + (int64_t)blockIdx.y * stride;
-  a[col + (int64_t)p * ld] = a[p + (int64_t)col * ld];
-}
-
 __global__ void zero_border_kernel(int j, double* Z, int64_t ld) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q > j) return;
@@ -69,14 +62,6 @@ __global__ void mask_residual_kernel(int64_t tot, int n, const double* __restric
   if (t >= tot) return;
   const int64_t i = t % n, a = t / n;
   E[t] = OmY[t] - (double)Om[i + a * ldo] * E[t];
-}
-
-__global__ void omega_times_kernel(int64_t tot, int n, const uint8_t* __restrict__ Om, int64_t ldo,
-                                   const double* __restrict__ u, double* B) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= tot) return;
-  const int64_t i = t % n, a = t / n;
-  B[t] = (double)Om[i + a * ldo] * u[i];
 }
 
 __global__ void mat_dot_kernel(int r, int c, const double* __restrict__ A, int64_t lda, const double* __restrict__ B,
@@ -164,12 +149,6 @@ void zcoef(int j, const double* Z, int64_t ldz, int trans, const double* h, doub
   zcoef_kernel<<<nblk(3 * j, 128), 128, 0, st>>>(j, Z, ldz, trans, h, lam, g);
 }
 
-void mirror_col(int col, double* A, int64_t ld, int batch, int64_t stride, cudaStream_t st) {
-  if (col <= 0 || batch <= 0) return;
-  count_launch();
-  mirror_col_kernel<<<dim3(nblk(col, 128), batch), 128, 0, st>>>(col, A, ld, stride);
-}
-
 void zero_border(int j, double* Z, int64_t ld, cudaStream_t st) {
   count_launch();
   zero_border_kernel<<<nblk(j + 1, 128), 128, 0, st>>>(j, Z, ld);
@@ -180,13 +159,6 @@ void mask_residual(int n, int m, const double* OmY, const uint8_t* Om, int64_t l
   if (tot == 0) return;
   count_launch();
   mask_residual_kernel<<<nblk(tot), 256, 0, st>>>(tot, n, OmY, Om, ldo, E);
-}
-
-void omega_times(int n, int m, const uint8_t* Om, int64_t ldo, const double* u, double* B, cudaStream_t st) {
-  const int64_t tot = (int64_t)n * m;
-  if (tot == 0) return;
-  count_launch();
-  omega_times_kernel<<<nblk(tot), 256, 0, st>>>(tot, n, Om, ldo, u, B);
 }
 
 void mat_dot(int r, int c, const double* A, int64_t lda, const double* B, int64_t ldb, double* out, cudaStream_t st) {
