@@ -451,20 +451,32 @@ cr_status check_csr(const cr_csr& c, int64_t n, const char* name, std::string& e
       return CR_EINVAL;
     }
   }
-  // symmetry: compare the entry list with its transpose
-  std::vector<std::tuple<int32_t, int32_t, double>> a, b;
-  const int64_t nnz = c.rowptr[n];
-  a.reserve(nnz);
-  b.reserve(nnz);
+  // symmetry: the entries by row (sorted within each row) against those of the transpose, which a
+  // counting pass over the sorted rows leaves in the same order
+  std::vector<int64_t> rp(n + 1, 0), at(n + 1, 0);
   for (int64_t i = 0; i < n; ++i)
     for (int32_t q = c.rowptr[i]; q < c.rowptr[i + 1]; ++q)
       if (c.val[q] != 0.0) {
-        a.emplace_back((int32_t)i, c.col[q], c.val[q]);
-        b.emplace_back(c.col[q], (int32_t)i, c.val[q]);
+        ++rp[i + 1];
+        ++at[c.col[q] + 1];
       }
-  std::sort(a.begin(), a.end());
-  std::sort(b.begin(), b.end());
-  if (a != b) {
+  for (int64_t i = 0; i < n; ++i) {
+    rp[i + 1] += rp[i];
+    at[i + 1] += at[i];
+  }
+  bool sym = rp == at;
+  if (sym) {
+    std::vector<std::pair<int32_t, double>> a((size_t)rp[n]), b((size_t)rp[n]);
+    for (int64_t i = 0; i < n; ++i) {
+      int64_t k = rp[i];
+      for (int32_t q = c.rowptr[i]; q < c.rowptr[i + 1]; ++q)
+        if (c.val[q] != 0.0) a[k++] = {c.col[q], c.val[q]};
+      std::sort(a.begin() + rp[i], a.begin() + rp[i + 1]);
+      for (k = rp[i]; k < rp[i + 1]; ++k) b[at[a[k].first]++] = {(int32_t)i, a[k].second};
+    }
+    sym = a == b;
+  }
+  if (!sym) {
     err = std::string(name) + ": matrix is not symmetric";
     return CR_EINVAL;
   }
@@ -858,16 +870,10 @@ cr_status build_mg_grid(cr_problem* p, const DevLap& L, const cr_mg::Hierarchy& 
   return CR_OK;
 }
 
-// Multigrid hierarchy of one Laplacian (cr_mg_host.h) on the cluster partition
-// of L: level 0 in L's chunks, larger coarse levels in equal chunks over the
-// cluster, levels of at most kMgTailRows rows and the coarsest (at most
-// kMgCoarseMax rows, through the eigenbasis of its pencil) on CTA 0.  Leaves
-// g.nlev = 0 when the hierarchy or its shared memory does not fit.
-cr_status build_mg(cr_problem* p, const cr_csr& c, const DevLap& L, DevMg& g) {
-  g = DevMg{};
+// Multigrid hierarchy of one Laplacian; empty where it has none (too few rows, or too many for a cluster).
+cr_mg::Hierarchy mg_hierarchy(const cr_csr& c, const DevLap& L) {
   const int n = (int)c.n;
-  const int C = L.csize;
-  if (C < 1 || n <= kMgCoarseMax) return CR_OK;
+  if (L.csize < 1 || n <= kMgCoarseMax) return cr_mg::Hierarchy{};
   cr_mg::Csr A;
   A.rows = A.cols = n;
   A.rp.assign(n + 1, 0);
@@ -886,7 +892,18 @@ cr_status build_mg(cr_problem* p, const cr_csr& c, const DevLap& L, DevMg& g) {
     }
     A.rp[i + 1] = (int)A.ci.size();
   }
-  const cr_mg::Hierarchy H = cr_mg::build(A, kMgCoarseMax, kMgMaxLev);
+  return cr_mg::build(A, kMgCoarseMax, kMgMaxLev);
+}
+
+// Multigrid hierarchy of one Laplacian (cr_mg_host.h) on the cluster partition
+// of L: level 0 in L's chunks, larger coarse levels in equal chunks over the
+// cluster, levels of at most kMgTailRows rows and the coarsest (at most
+// kMgCoarseMax rows, through the eigenbasis of its pencil) on CTA 0.  Leaves
+// g.nlev = 0 when the hierarchy or its shared memory does not fit.
+cr_status build_mg(cr_problem* p, const cr_mg::Hierarchy& H, const DevLap& L, DevMg& g) {
+  g = DevMg{};
+  const int n = L.n;
+  const int C = L.csize;
   const int nlev = (int)H.lev.size();
   if (nlev < 2 || H.lev.back().L.rows > kMgCoarseMax) return CR_OK;
   double bytes_iter[2];
@@ -2276,7 +2293,15 @@ cr_status cr_create(const cr_problem_desc* d_in, const cr_options* o, cr_problem
     return bad("galerkin_form must be a cr_galerkin_form");
   if (opt.alloc && !opt.free) return bad("alloc given without free");
   std::string err;
-  if (check_csr(d->Lx, nx, "Lx", err) != CR_OK || check_csr(d->Ly, ny, "Ly", err) != CR_OK) return bad(err);
+  if (check_csr(d->Lx, nx, "Lx", err) != CR_OK) return bad(err);
+  // one Laplacian for both grids (source and target voxels are the same): its checks and set-up serve both
+  const bool one_grid =
+      nx == ny && d->Ly.n == d->Lx.n && d->Ly.rowptr && d->Ly.col && d->Ly.val &&
+      (d->Ly.rowptr == d->Lx.rowptr ||
+       std::memcmp(d->Ly.rowptr, d->Lx.rowptr, sizeof(int32_t) * (nx + 1)) == 0) &&
+      (d->Ly.col == d->Lx.col || std::memcmp(d->Ly.col, d->Lx.col, sizeof(int32_t) * d->Lx.rowptr[nx]) == 0) &&
+      (d->Ly.val == d->Lx.val || std::memcmp(d->Ly.val, d->Lx.val, sizeof(double) * d->Lx.rowptr[nx]) == 0);
+  if (!one_grid && check_csr(d->Ly, ny, "Ly", err) != CR_OK) return bad(err);
   if (d->grid_x.box_index && !grid_ok(d->grid_x.dims, d->grid_x.box_index, nx, err)) return bad("grid_x: " + err);
   if (d->grid_y.box_index && !grid_ok(d->grid_y.dims, d->grid_y.box_index, ny, err)) return bad("grid_y: " + err);
   for (int64_t a = 0; a < m; ++a) {
@@ -2320,12 +2345,19 @@ cr_status cr_create(const cr_problem_desc* d_in, const cr_options* o, cr_problem
     if ((s = (x)) != CR_OK) return abort_create(s); \
   } while (0)
   CK(build_lap(p, d->Ly, p->Ly));
-  CK(build_lap(p, d->Lx, p->Lx));
+  if (one_grid) {
+    p->Lx = p->Ly;
+    p->push[1] = p->push[0];
+  } else {
+    CK(build_lap(p, d->Lx, p->Lx));
+  }
   if (opt.precond == CR_PRECOND_MULTIGRID || opt.precond == CR_PRECOND_AUTO) {
-    CK(build_mg(p, d->Ly, p->Ly, p->mg[0]));
-    CK(build_mg(p, d->Lx, p->Lx, p->mg[1]));
+    const cr_mg::Hierarchy H = mg_hierarchy(d->Ly, p->Ly);
+    CK(build_mg(p, H, p->Ly, p->mg[0]));
+    CK(build_mg(p, one_grid ? H : mg_hierarchy(d->Lx, p->Lx), p->Lx, p->mg[1]));
   }
   // X: CSC, CSR by rows, and per-CTA local CSC on the x partition
+  std::vector<int> xbeg(m), xnnz(m);  // first entry and entries of each column
   {
     std::vector<int> cp(m + 1, 0), row;
     std::vector<double> val;
@@ -2340,6 +2372,8 @@ cr_status cr_create(const cr_problem_desc* d_in, const cr_options* o, cr_problem
         }
       }
       cp[a + 1] = (int)row.size();
+      xbeg[a] = cp[a];
+      xnnz[a] = cp[a + 1] - cp[a];
     }
     std::vector<int> rp(nx + 1, 0), rc;
     std::vector<double> rv;
@@ -2387,8 +2421,7 @@ cr_status cr_create(const cr_problem_desc* d_in, const cr_options* o, cr_problem
       p->mg[1].xn2 = dx;
     }
   }
-  // Omega o Y, Omega; norms |D|_F (via the m x m Gram products, all terms of
-  // one sign pattern: |D|^2 = tr((OmY^T OmY)(X^T X))) and |Omega o Y|^2
+  // Omega o Y, Omega
   std::vector<double> omy((size_t)ny * m);
   std::vector<uint8_t> om((size_t)ny * m);
   for (int64_t a = 0; a < m; ++a)
@@ -2396,22 +2429,6 @@ cr_status cr_create(const cr_problem_desc* d_in, const cr_options* o, cr_problem
       om[i + a * ny] = d->Omega_host[i + a * d->ldo];
       omy[i + a * ny] = om[i + a * ny] ? d->Y_host[i + a * d->ldy] : 0.0;
     }
-  {
-    std::vector<double> g1((size_t)m * m, 0.0), g2((size_t)m * m, 0.0);
-    for (int64_t a = 0; a < m; ++a)
-      for (int64_t b = 0; b <= a; ++b) {
-        double s1 = 0.0, s2 = 0.0;
-        for (int64_t i = 0; i < ny; ++i) s1 += omy[i + a * ny] * omy[i + b * ny];
-        for (int64_t i = 0; i < nx; ++i) s2 += d->X_host[i + a * d->ldx] * d->X_host[i + b * d->ldx];
-        g1[a + b * m] = g1[b + a * m] = s1;
-        g2[a + b * m] = g2[b + a * m] = s2;
-      }
-    double dn2 = 0.0, on2 = 0.0;
-    for (size_t t = 0; t < g1.size(); ++t) dn2 += g1[t] * g2[t];
-    for (int64_t a = 0; a < m; ++a) on2 += g1[a + a * m];
-    p->Dnorm = std::sqrt(std::max(dn2, 0.0));
-    p->OmYn2 = on2;
-  }
   {
     std::vector<int> zp(m + 1, 0), zr;
     std::vector<uint8_t> full(m, 0);
@@ -2519,42 +2536,75 @@ cr_status cr_create(const cr_problem_desc* d_in, const cr_options* o, cr_problem
   p->ws_elems = std::max<size_t>((size_t)8 * p->ldcp * p->ldm, (size_t)16 * (3 * rc + m) * m);
   p->ws_elems = std::max<size_t>(std::max<size_t>(p->ws_elems, (size_t)16 * r2), 1024);
   CK(dalloc(p, &p->ws, p->ws_elems));
-  // right residual basis: X first (host Gram-Schmidt twice, columns in X's span rejected)
+  // right residual basis: X first (Gram-Schmidt twice, columns in X's span rejected), and the
+  // coefficients C of X's columns in it; |Omega o Y|^2, and |D|_F from
+  // |D|^2 = tr((OmY^T OmY)(X^T X)) with X^T X = C^T C.  On the device a column costs nine launches
+  // and a read-back, 50 us, on the host 2 m nx FMAs on average: the host is the quicker one up to
+  // m nx = 25,000 (a whole creation on a 20 x 20 grid, 5 injections: 1.6 ms, 1.9 on the device; on
+  // 15,000 voxels, 126 injections: 55 ms, 620 on the host with two set-ups of the one grid)
   {
-    std::vector<double> Q((size_t)nx * m, 0.0), Cm((size_t)p->ldcr * m, 0.0);
+    const bool on_host = m * std::max(nx, ny) <= 25000;
+    std::vector<double> g1((size_t)m * m), C((size_t)p->ldcr * m, 0.0);
     int nq = 0;
-    std::vector<double> w(nx);
-    for (int64_t a = 0; a < m; ++a) {
-      for (int64_t i = 0; i < nx; ++i) w[i] = d->X_host[i + a * d->ldx];
-      double nb = 0.0;
-      for (double x : w) nb += x * x;
-      for (int pass = 0; pass < 2; ++pass)
-        for (int q = 0; q < nq; ++q) {
-          double c = 0.0;
-          for (int64_t i = 0; i < nx; ++i) c += Q[i + (size_t)q * nx] * w[i];
-          for (int64_t i = 0; i < nx; ++i) w[i] -= c * Q[i + (size_t)q * nx];
-        }
-      double na = 0.0;
-      for (double x : w) na += x * x;
-      if (nb > 0.0 && std::sqrt(na / nb) > 1e-12) {
+    if (on_host) {
+      std::vector<double> Q((size_t)nx * m, 0.0), w(nx);
+      auto hdot = [](int64_t n, const double* x, const double* y) {
+        double t = 0.0;
+        for (int64_t i = 0; i < n; ++i) t += x[i] * y[i];
+        return t;
+      };
+      for (int64_t a = 0; a < m; ++a) {
+        const double* x = d->X_host + a * d->ldx;
+        std::copy(x, x + nx, w.begin());
+        for (int pass = 0; pass < 2; ++pass)
+          for (int q = 0; q < nq; ++q) {
+            const double* Qq = Q.data() + (size_t)q * nx;
+            const double c = hdot(nx, Qq, w.data());
+            for (int64_t i = 0; i < nx; ++i) w[i] -= c * Qq[i];
+          }
+        const double nb = hdot(nx, x, x), na = hdot(nx, w.data(), w.data());
+        if (!(nb > 0.0 && std::sqrt(na / nb) > 1e-12)) continue;
         const double inv = 1.0 / std::sqrt(na);
         for (int64_t i = 0; i < nx; ++i) Q[i + (size_t)nq * nx] = w[i] * inv;
         ++nq;
       }
-    }
-    for (int64_t a = 0; a < m; ++a)
-      for (int q = 0; q < nq; ++q) {
-        double c = 0.0;
-        for (int64_t i = 0; i < nx; ++i) c += Q[i + (size_t)q * nx] * d->X_host[i + a * d->ldx];
-        Cm[q + (size_t)a * p->ldcr] = c;
+      for (int64_t a = 0; a < m; ++a) {
+        for (int q = 0; q < nq; ++q) C[q + a * p->ldcr] = hdot(nx, Q.data() + (size_t)q * nx, d->X_host + a * d->ldx);
+        for (int64_t b = 0; b <= a; ++b) g1[a + b * m] = hdot(ny, omy.data() + a * ny, omy.data() + b * ny);
       }
-    CUCHK(p, cudaMemcpyAsync(p->QR, Q.data(), sizeof(double) * nx * nq, cudaMemcpyHostToDevice, p->st));
-    p->h2d_bytes += (int64_t)(sizeof(double) * nx * nq);
-    CUCHK(p, cudaMemcpyAsync(p->CRm, Cm.data(), sizeof(double) * Cm.size(), cudaMemcpyHostToDevice, p->st));
-    p->h2d_bytes += (int64_t)(sizeof(double) * Cm.size());
+      CUCHK(p, cudaMemcpyAsync(p->QR, Q.data(), sizeof(double) * nx * nq, cudaMemcpyHostToDevice, p->st));
+      CUCHK(p, cudaMemcpyAsync(p->CRm, C.data(), sizeof(double) * C.size(), cudaMemcpyHostToDevice, p->st));
+      p->h2d_bytes += (int64_t)(sizeof(double) * (nx * nq + C.size()));
+    } else {
+      for (int64_t a = 0; a < m; ++a) {
+        double* dst = p->QR + (size_t)nq * nx;
+        fill(nx, 0.0, dst, p->st);
+        scatter_col(xnnz[a], p->xc_row + xbeg[a], p->xc_val + xbeg[a], dst, p->st);
+        double ratio = 0.0;
+        if (xnnz[a] > 0) CK(cgs2(p, (int)nx, p->QR, nx, nq, dst, &ratio));
+        if (ratio > 1e-12) ++nq;
+      }
+      sparse_cols_t((int)m, nq, p->QR, nx, p->xc_ptr, p->xc_row, p->xc_val, p->CRm, p->ldcr, p->st);
+      gemm((int)m, (int)m, (int)ny, 1.0, MatView{p->OmY, ny, 1}, MatView{p->OmY, 1, ny}, 0.0, p->gram, 1, m, p->ws,
+           p->ws_elems, p->st);
+      CUCHK(p, cudaMemcpyAsync(g1.data(), p->gram, sizeof(double) * m * m, cudaMemcpyDeviceToHost, p->st));
+      CUCHK(p, cudaMemcpyAsync(C.data(), p->CRm, sizeof(double) * C.size(), cudaMemcpyDeviceToHost, p->st));
+      p->d2h_bytes += (int64_t)(sizeof(double) * (g1.size() + C.size()));
+    }
+    if ((s = sync(p)) != CR_OK) return abort_create(s);
+    double dn2 = 0.0, on2 = 0.0;
+    for (int64_t a = 0; a < m; ++a) {
+      on2 += g1[a + a * m];
+      for (int64_t b = 0; b <= a; ++b) {
+        double x = 0.0;
+        for (int q = 0; q < nq; ++q) x += C[q + a * p->ldcr] * C[q + b * p->ldcr];
+        dn2 += (b < a ? 2.0 : 1.0) * g1[a + b * m] * x;
+      }
+    }
+    p->Dnorm = std::sqrt(std::max(dn2, 0.0));
+    p->OmYn2 = on2;
     p->nQR = nq;
     p->nQX = nq;
-    if (sync(p) != CR_OK) return abort_create(CR_ECUDA);
   }
   refresh_E(p);
   if ((s = sync(p)) != CR_OK) return abort_create(s);

@@ -220,6 +220,28 @@ __global__ void spmv_xt_kernel(int m, const int* __restrict__ cp, const int* __r
   if (lane == 0) out[(int64_t)a * ostride] = acc;
 }
 
+// y[row[k]] = val[k], k < nnz
+__global__ void scatter_kernel(int nnz, const int* __restrict__ row, const double* __restrict__ val,
+                               double* __restrict__ y) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < nnz) y[row[k]] = val[k];
+}
+
+// C(q, a) = Q(:, q)^T X_a, one warp per entry
+__global__ void sparse_cols_t_kernel(int m, int nq, const double* __restrict__ Q, int64_t ldq, const int* __restrict__ cp,
+                                     const int* __restrict__ row, const double* __restrict__ val, double* __restrict__ C,
+                                     int64_t ldc) {
+  const int lane = threadIdx.x & 31;
+  const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (t >= (int64_t)m * nq) return;
+  const int q = (int)(t % nq), a = (int)(t / nq);
+  const double* c = Q + q * ldq;
+  double acc = 0.0;
+  for (int p = cp[a] + lane; p < cp[a + 1]; p += 32) acc = fma(val[p], c[row[p]], acc);
+  acc = warp_sum(acc);
+  if (lane == 0) C[q + a * ldc] = acc;
+}
+
 __global__ void spmv_x_kernel(int n, const int* __restrict__ rp, const int* __restrict__ col,
                               const double* __restrict__ val, const double* __restrict__ c, double* y, double alpha,
                               double beta) {
@@ -374,6 +396,20 @@ void spmv_xt(int m, const int* colptr, const int* row, const double* val, const 
   if (m <= 0) return;
   count_launch();
   spmv_xt_kernel<<<(m + 7) / 8, 256, 0, st>>>(m, colptr, row, val, v, out, ostride);
+}
+
+void scatter_col(int nnz, const int* row, const double* val, double* y, cudaStream_t st) {
+  if (nnz <= 0) return;
+  count_launch();
+  scatter_kernel<<<(nnz + 255) / 256, 256, 0, st>>>(nnz, row, val, y);
+}
+
+void sparse_cols_t(int m, int nq, const double* Q, int64_t ldq, const int* cp, const int* row, const double* val, double* C,
+                   int64_t ldc, cudaStream_t st) {
+  const int64_t t = (int64_t)m * nq;
+  if (t <= 0) return;
+  count_launch();
+  sparse_cols_t_kernel<<<(unsigned)((t + 7) / 8), 256, 0, st>>>(m, nq, Q, ldq, cp, row, val, C, ldc);
 }
 
 void spmv_x(int n, const int* rowptr, const int* col, const double* val, const double* c, double* y, double alpha,

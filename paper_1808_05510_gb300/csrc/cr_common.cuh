@@ -326,6 +326,11 @@ void spmv_xt(int m, const int* colptr, const int* row, const double* val, const 
 // y[k] = beta*y[k] + alpha * sum_a X_ka * c[a], X by rows (CSR)
 void spmv_x(int n, const int* rowptr, const int* col, const double* val, const double* c, double* y,
             double alpha, double beta, cudaStream_t st);
+// y[row[k]] = val[k], k < nnz
+void scatter_col(int nnz, const int* row, const double* val, double* y, cudaStream_t st);
+// C(q, a) = Q(:, q)^T X_a for q < nq, a < m, X by columns
+void sparse_cols_t(int m, int nq, const double* Q, int64_t ldq, const int* cp, const int* row, const double* val, double* C,
+                   int64_t ldc, cudaStream_t st);
 // out[a] = sum_i Om[i + a*ldo] * u[i]^2
 void omega_sq_dots(int n, int m, const uint8_t* Om, int64_t ldo, const double* u, double* out,
                    cudaStream_t st);
