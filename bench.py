@@ -156,7 +156,8 @@ def peaks():
         return 6800.0, "of fallback"
 
 
-KERNEL_SOURCES = {"pcg_reg_kernel": "cr_pcg.cu", "pcg_mg_kernel": "cr_mg.cu", "pcg_grid_kernel": "cr_pcg_grid.cu"}
+KERNEL_SOURCES = {"pcg_reg_kernel": "cr_pcg.cu", "pcg_push_kernel": "cr_pcg_push.cu", "pcg_mg_kernel": "cr_mg.cu",
+                  "pcg_mg_grid_kernel": "cr_mg_grid.cu", "pcg_grid_kernel": "cr_pcg_grid.cu"}
 
 
 def pcg_traffic(kernel: str, form: str, side: int):
@@ -315,8 +316,12 @@ def run_ours(args, rank, world, local_rank):
             ipl = its / calls
             avg_s = kms / calls / 1e3
             bpi = stats["pcg_bytes_per_iter"][side]
-            kname = ("pcg_mg_kernel" if stats["pcg_multigrid"][side] else
-                     "pcg_reg_kernel" if stats["pcg_cluster"][side] else "pcg_grid_kernel")
+            cluster = stats["pcg_cluster"][side] > 0
+            if stats["pcg_multigrid"][side]:
+                kname = "pcg_mg_kernel" if cluster else "pcg_mg_grid_kernel"
+            else:
+                kname = ("pcg_grid_kernel" if not cluster else
+                         "pcg_push_kernel" if prec == CR_MIXED else "pcg_reg_kernel")
             sides.append({"side": "uv"[side], "kernel": kname, "kernel_ms_per_step": kms / steps, "launches": calls,
                           "iters": its, "iters_per_launch": ipl, "avg_launch_us": avg_s * 1e6,
                           "us_per_iter": avg_s * 1e6 / max(ipl, 1e-9), "bytes_per_iter": bpi,

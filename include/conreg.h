@@ -56,8 +56,9 @@ typedef enum { CR_FP64 = 0, CR_MIXED = 1 } cr_precision;
  * of lam (L + sigma I)^2, sigma^2 = the Laplacian shift plus the mean data
  * weight over lam), hierarchy built once from L at cr_create; on the v side
  * with at most 32 injections the data term is added exactly by
- * Sherman-Morrison-Woodbury; sizes whose vectors do not fit one thread-block
- * cluster fall back to Jacobi.  CR_PRECOND_AUTO: multigrid in the float64
+ * Sherman-Morrison-Woodbury.  It runs on all SMs, or in one thread-block
+ * cluster when cluster_size or galerkin_ctas is set (members of a sweep share
+ * the GPU); grids beyond one cluster's rows fall back to Jacobi.  CR_PRECOND_AUTO: multigrid in the float64
  * form; in the mixed form multigrid above 20,000 rows or for lambda >= 1e3
  * (where the Laplacian term dominates and Jacobi's iteration count grows),
  * Jacobi otherwise (there its many cheap float32 iterations are faster). */
@@ -151,10 +152,10 @@ typedef struct {
                               (1 to 32), so sparse far from it and every step close to it */
   int32_t cluster_size;    /* PCG thread-block cluster size; 0 = automatic */
   int32_t profile;         /* != 0: time each phase with CUDA events (see cr_get_stats) */
-  int32_t pcg_kernel;      /* 0 = automatic: the register-resident cluster kernel (the whole solve on
-                              chip) while it applies (unit-weight Laplacian, at most 6 neighbours per
-                              row, up to 1,024 rows per CTA in float64 or 2,048 in float32), else the
-                              grid-wide kernel; 1 = the generic cluster kernel (grids that fit one
+  int32_t pcg_kernel;      /* 0 = automatic: a register-resident cluster kernel (the whole solve on
+                              chip, float32 values pushed between the CTAs) while it applies (unit-weight
+                              Laplacian, at most 6 neighbours per row, up to 1,024 rows per CTA in float64
+                              or 2,048 in float32), else the grid-wide kernel; 1 = the generic cluster kernel (grids that fit one
                               cluster); 2 = always the grid-wide kernel */
   int32_t galerkin_kernel; /* 0 = one persistent cooperative launch per projection, 1 = one launch per step */
   uint64_t seed;           /* seed of the fallback ALS start vector */
@@ -223,7 +224,7 @@ typedef struct {
   int64_t learned_off;            /* bit s set: the learned form is switched off for side s */
   int64_t mixed_handovers;        /* mixed-form sub-solves that float32 refinement handed to float64 */
   int64_t pcg_cluster[2];         /* CTAs per thread-block cluster of the u-side (0) and v-side (1) PCG;
-                                     0 = the grid-wide kernel */
+                                     0 = a grid-wide kernel (Jacobi or multigrid) */
   int64_t pcg_multigrid[2];       /* levels of the multigrid preconditioner per side (0 = not in use) */
   int64_t galerkin_eigen[2];      /* projections solved in the eigenbasis form (0), of which the
                                      original-basis CG had to finish (1) */
