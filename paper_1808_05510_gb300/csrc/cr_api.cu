@@ -1443,8 +1443,8 @@ cr_status launch_pcg_mixed(cr_problem* p, int side, const double* b, double* x, 
     rr_prev = rr;
     fill(n, 0.0, d, st);
     // an inner solve never goes further than the float64 target needs (with a
-    // factor 2 to spare): on warm-started sweeps the last step is much shorter
-    const double inner = std::max(kMixedInnerTol, 0.5 * std::sqrt(tol * tol * bb / rr));
+    // factor 4 to spare): on warm-started sweeps the last step is much shorter
+    const double inner = std::max(kMixedInnerTol, 0.25 * std::sqrt(tol * tol * bb / rr));
     TRY(run_pcg(p, side, r, d, maxit - total, inner, true));
     TRY(readback(p, 0, 1, true));
     const PcgStat in = p->hs->stat[side];
