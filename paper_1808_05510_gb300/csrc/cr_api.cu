@@ -860,10 +860,7 @@ cr_status build_mg_grid(cr_problem* p, const DevLap& L, const cr_mg::Hierarchy& 
   d.rc = rc;
   TRY(dalloc(p, &d.ytot, (size_t)m));
   TRY(dalloc(p, &d.part, (size_t)4 * d.nb));
-  if (h.smw) {
-    TRY(dalloc(p, &d.smw_lmx, (size_t)n * m));
-    TRY(dalloc(p, &d.smw_rows, (size_t)3 * n * m));
-  }
+  if (h.smw) TRY(dalloc(p, &d.smw_rows, (size_t)n * m));
   TRY(dalloc(p, &d.bar, 2));
   d.err = reinterpret_cast<int*>(d.bar + 1);
   out = d;

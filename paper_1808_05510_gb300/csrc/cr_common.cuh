@@ -236,8 +236,7 @@ struct DevMgGrid {
   char* tab_glob = nullptr;
   void* rc = nullptr;         // coarsest right side
   double *ytot = nullptr, *part = nullptr;
-  double* smw_lmx = nullptr;   // v side, smw: L MX, beside DevMg::smw_mx
-  double* smw_rows = nullptr;  // v side, smw: per row [MX Q | (L + cI) MX Q | X Q] (3 m values of the working precision)
+  double* smw_rows = nullptr;  // v side, smw: rows of MX Q (m values of the working precision each), beside DevMg::smw_mx
   unsigned* bar = nullptr;  // the barrier's counter, then its error word
   int* err = nullptr;
   const int *xc_ptr = nullptr, *xc_row = nullptr;  // v side: X by columns (set at the launch)

@@ -14,7 +14,8 @@
 //    two phases down and two up per level instead of three and three.  On the
 //    level above the coarsest, S times the coarsest inverse is formed once per
 //    launch (own rows x nc, dense), which leaves no coarse-solve phase.  A
-//    three-level PCG iteration takes 19 barriers (the cluster kernel: 28).
+//    three-level PCG iteration takes 19 barriers (the cluster kernel: 28), two more
+//    with the v side's Woodbury step.
 //  - All SMs.  The float64 pipe of GB300 issues one warp operation per 16 cycles,
 //    so a level-0 sweep over 470 rows per CTA (16-CTA cluster, 7,530 voxels) is
 //    1.2 us of float64 arithmetic alone; 152 CTAs hold 50 rows each, and every
@@ -25,9 +26,8 @@
 // in a fixed order and every CTA forms the same scalars, so results repeat bit for
 // bit and all CTAs take the same branches.
 // Measured against the cluster kernel (ms per solve): 7,500 voxels, float64, v side
-// with 28 injections 2.93 -> 1.79; 45,000 voxels, float32, u side 6.42 -> 2.26.  An
-// iteration at 7,500 voxels in float64 is 102 -> 47 us: 19 barriers of 1.2 us and 24 us
-// between them.
+// with 28 injections 2.92 -> 1.91; 45,000 voxels, float32, u side 6.42 -> 2.26.  An
+// iteration of that v side is 102 -> 50 us: 21 barriers of 1.2 us and 25 us between them.
 #include <algorithm>
 
 #include "cr_common.cuh"
@@ -494,7 +494,6 @@ __global__ void __launch_bounds__(kMgGridThreads, 1) pcg_mg_grid_kernel(const Pc
 
   // ---- v side: Sherman-Morrison-Woodbury correction (see cr_mg.cu) ----------------------
   T* const mx = reinterpret_cast<T*>(G.smw_mx);
-  T* const lmx = reinterpret_cast<T*>(D.smw_lmx);  // L MX, formed with MX
   if (smw) {
     if (smw_build) {
       for (int a = 0; a < m; ++a) {
@@ -511,15 +510,6 @@ __global__ void __launch_bounds__(kMgGridThreads, 1) pcg_mg_grid_kernel(const Pc
         vcycle(false, [&](int li, T y) { mx[(size_t)(beg0 + li) * m + a] = ilam * y; });
       }
       gsync();
-      for (int idx = tid; idx < n0 * m; idx += nth) {
-        const int li = idx / m, a = idx % m;
-        T acc = DG[li] * mx[(size_t)(beg0 + li) * m + a];
-        for (int k = 0; k < K; ++k) {
-          const int jn = nbt[k * ch0 + li];
-          if (jn >= 0) acc += (nbw ? nbw[k * ch0 + li] : (T)-1) * __ldcg(mx + (size_t)jn * m + a);
-        }
-        lmx[(size_t)(beg0 + li) * m + a] = acc;
-      }
       // X^T MX: column a of X against every column of MX
       for (int a = b; a < m; a += nb) {
         const int p0 = D.xc_ptr[a], p1 = D.xc_ptr[a + 1];
@@ -564,60 +554,46 @@ __global__ void __launch_bounds__(kMgGridThreads, 1) pcg_mg_grid_kernel(const Pc
     for (int idx = tid; idx < m * m; idx += nth)
       smw_ci[idx] *= sqrt(fmax(sS[idx / m], 0.0)) * sqrt(fmax(sS[idx % m], 0.0));  // Q = D C^-1 D
     __syncthreads();
-    // With y = X^T u0 (u0 = M0^-1 r) and g = Q y: u = u0 - MX g, t = (L + cI) u = t0 - (L + cI) MX g,
-    // and the data term X S X^T u = X g, because S (X^T u0 - X^T MX g) = D (I - D X^T MX D C^-1) D y
-    // = D C^-1 D y.  The three row products are formed here for the own rows, so that an iteration
-    // needs y alone: the correction shares the operator's phase instead of taking two of its own.
-    // (MX and L MX of the own rows: written by this CTA, so ordinary loads see them.)
+    // With y = X^T u0 (u0 = M0^-1 r) the correction is u = u0 - MX Q y: the rows of MX Q are formed
+    // here for the own rows (MX of the own rows was written by this CTA, so ordinary loads see it).
+    // The operator is then applied to the u that enters x.  Its data term also follows from y
+    // (S X^T u = Q y), and t from stored rows of (L + cI) MX Q, which would save a phase, but in the
+    // span of X u0 is much larger than u, and A u then differs from that of the rounded u by u0's
+    // rounding: solves for 1e-13 stopped at 1e-12 of the right side, float32 ones for 1e-5 at 1e-4.
     for (int idx = tid; idx < n0 * m; idx += nth) {
       const int li = idx / m, q = idx % m, i = beg0 + li;
-      const T *r1 = mx + (size_t)i * m, *r2 = lmx + (size_t)i * m;
-      double s1 = 0.0, s2 = 0.0, s3 = 0.0;
+      const T* row = mx + (size_t)i * m;
+      double acc = 0.0;
 #pragma unroll 4
-      for (int a = 0; a < m; ++a) {
-        const double qa = smw_ci[a * m + q];
-        s1 += (double)r1[a] * qa;
-        s2 += (double)r2[a] * qa;
-      }
-      for (int p = A.X.xr_ptr[i]; p < A.X.xr_ptr[i + 1]; ++p) s3 += A.X.xr_val[p] * smw_ci[A.X.xr_col[p] * m + q];
-      T* o = reinterpret_cast<T*>(D.smw_rows) + (size_t)3 * i * m + q;
-      o[0] = (T)s1;
-      o[m] = (T)(s2 + c * s1);
-      o[2 * m] = (T)s3;
+      for (int a = 0; a < m; ++a) acc += (double)row[a] * smw_ci[a * m + q];
+      reinterpret_cast<T*>(D.smw_rows)[(size_t)i * m + q] = (T)acc;
     }
     __syncthreads();
   }
-  // after a barrier behind op_t(u0): u, t (published) and the data term in W0 of the own rows
+  // after the barrier behind u0 (published): the corrected u of the own rows, published
   auto smw_correct = [&]() {
+    xt_cols(gu);
+    gsync();
     for (int a = tid; a < m; a += nth) sY[a] = __ldcg(D.ytot + a);
     __syncthreads();
-    // two lanes per row: the float64 pipe bounds this (three products of m a row), and sums over
-    // more lanes would add to its work
+    // two lanes per row: sums over more lanes would add to the float64 pipe's work
     const int ln = tid % 2, rpp = nth / 2;
     for (int base = 0; base < n0; base += rpp) {
       const int li = base + tid / 2;
-      T a1 = (T)0, a2 = (T)0, a3 = (T)0;
+      T acc = (T)0;
       if (li < n0) {
-        const T* row = reinterpret_cast<const T*>(D.smw_rows) + (size_t)3 * (beg0 + li) * m;
+        const T* row = reinterpret_cast<const T*>(D.smw_rows) + (size_t)(beg0 + li) * m;
 #pragma unroll 4
-        for (int q = ln; q < m; q += 2) {
-          const T yq = (T)sY[q];
-          a1 += row[q] * yq;
-          a2 += row[m + q] * yq;
-          a3 += row[2 * m + q] * yq;
-        }
+        for (int q = ln; q < m; q += 2) acc += row[q] * (T)sY[q];
       }
-      a1 += __shfl_xor_sync(0xffffffffu, a1, 1);
-      a2 += __shfl_xor_sync(0xffffffffu, a2, 1);
-      a3 += __shfl_xor_sync(0xffffffffu, a3, 1);
+      acc += __shfl_xor_sync(0xffffffffu, acc, 1);
       if (li < n0 && ln == 0) {
-        const T t = TT[li] - a2;
-        TT[li] = t;
-        gt0[beg0 + li] = t;
-        U0[li] -= a1;
-        W0[li] = a3;
+        const T u = U0[li] - acc;
+        U0[li] = u;
+        gu[beg0 + li] = u;
       }
     }
+    gsync();
   };
 
   // ---- r0 = b - A x0 --------------------------------------------------------------------
@@ -681,18 +657,14 @@ __global__ void __launch_bounds__(kMgGridThreads, 1) pcg_mg_grid_kernel(const Pc
       gu[beg0 + li] = u;
     });
     gsync();
+    if (smw) smw_correct();
     op_t(U0);
     gsync();
-    if (smw) {
-      smw_correct();
-      gsync();
-    } else {
-      load_y();
-    }
+    load_y();
     double v[2] = {0.0, 0.0};
     for (int li = tid; li < n0; li += nth) {
       const T ui = U0[li];
-      const T wi = lamT * (lap0(li, gt0, TT[li], cT) + eT * ui) + (smw ? W0[li] : data(li, ui));
+      const T wi = lamT * (lap0(li, gt0, TT[li], cT) + eT * ui) + data(li, ui);
       W0[li] = wi;
       v[0] += (double)Rr[li] * (double)ui;
       v[1] += (double)ui * (double)wi;
