@@ -243,6 +243,8 @@ struct cr_problem {
   double* post_scale[4] = {nullptr, nullptr, nullptr, nullptr};
   int post_dig_cap[4] = {0, 0, 0, 0};
   int* post_odd = nullptr;
+  uint8_t* post_wide = nullptr;  // tiles that the digits do not hold
+  int64_t post_wide_cap = 0;
   int64_t post_part_cap = 0, post_W_cols = 0;
   int64_t fcg_fallbacks = 0, learned_solves = 0, mixed_handovers = 0;
   // grid-wide PCG (grids the register-resident kernel does not take, or pcg_kernel = 2): work buffers
@@ -3132,10 +3134,14 @@ cr_status cr_solution_report(cr_problem* p, int32_t nonneg, int32_t jr, const do
     }
   }
   // tensor-core form: digits of the four factors, and the float64 pass behind it for
-  // factors that they cannot hold
+  // the tiles that they do not hold
   const bool tc = j > 0 && (j + jr >= kPostTcRank || out->entries >= kPostTcEntries) && post_tc_blocks() > 0;
   if (tc) {
     if (!p->post_odd) TRY(dalloc(p, &p->post_odd, 1));
+    if ((int64_t)post_wide_tiles(ny, (int)cw) > p->post_wide_cap) {
+      p->post_wide_cap = (int64_t)post_wide_tiles(ny, (int)cw);
+      TRY(dalloc(p, &p->post_wide, (size_t)p->post_wide_cap));
+    }
     CUCHK(p, cudaMemsetAsync(p->post_odd, 0, sizeof(int), st));
     const double* src[4] = {p->post_P, p->VV, p->post_Pr, p->post_Vr};
     const int64_t lds[4] = {ny, 3 * (int64_t)nx, ny, nx};
@@ -3164,13 +3170,13 @@ cr_status cr_solution_report(cr_problem* p, int32_t nonneg, int32_t jr, const do
   for (int64_t c0 = 0; c0 < nx; c0 += cw) {
     const int ncols = (int)std::min<int64_t>(cw, nx - c0);
     if (tc) {
-      post_tc_tiles(p->post_odd, ny, nx, j, p->post_dig[0], p->post_scale[0], p->post_dig[1], p->post_scale[1], jr,
+      post_tc_tiles(p->post_odd, p->post_wide, ny, nx, j, p->post_dig[0], p->post_scale[0], p->post_dig[1], p->post_scale[1], jr,
                     p->post_dig[2], p->post_scale[2], p->post_dig[3], p->post_scale[3], nonneg ? 1 : 0, (int)c0, ncols,
                     W ? p->post_W : nullptr, ny, p->post_part + off * PS_N, st);
       off += post_tc_parts(ny, ncols);
     }
-    post_tiles(tc ? p->post_odd : nullptr, ny, j, p->post_P, ny, p->VV, 3 * (int64_t)nx, jr, p->post_Pr, ny, p->post_Vr, nx, nonneg ? 1 : 0,
-               (int)c0, ncols, W ? p->post_W : nullptr, ny, p->post_part + off * PS_N, st);
+    post_tiles(tc ? p->post_wide : nullptr, ny, j, p->post_P, ny, p->VV, 3 * (int64_t)nx, jr, p->post_Pr, ny, p->post_Vr, nx,
+               nonneg ? 1 : 0, (int)c0, ncols, W ? p->post_W : nullptr, ny, p->post_part + off * PS_N, st);
     off += post_tiles_parts(ny, ncols);
     if (W) {
       CUCHK(p, cudaMemcpy2DAsync(W + c0 * ldw, ldw * sizeof(double), p->post_W, ny * sizeof(double),

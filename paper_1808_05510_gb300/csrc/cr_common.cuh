@@ -483,20 +483,22 @@ int post_tiles_parts(int ny, int ncols);
 // Columns [col0, col0 + ncols) of W = P V^T (P = U Z: ny x j, ld ldp; V(c, k) at
 // V[c + k ldv]) against W* = Pr Vr^T (jr = 0: W* = 0); P(W) = max(0, W) if nonneg.
 // Writes post_tiles_parts(ny, ncols) rows of PS_N statistics to part, and P(W)
-// to out (column c at out + (c - col0) ldo) unless out is null.  run_if (may be
-// null): a device flag; where it is not set the pass leaves empty statistics.
-void post_tiles(const int* run_if, int ny, int j, const double* P, int64_t ldp, const double* V, int64_t ldv, int jr,
+// to out (column c at out + (c - col0) ldo) unless out is null.  only (may be null):
+// a byte per 64 x 64 tile (post_wide_tiles, row tile fastest); tiles where it is 0 are passed by.
+void post_tiles(const uint8_t* only, int ny, int j, const double* P, int64_t ldp, const double* V, int64_t ldv, int jr,
                 const double* Pr, int64_t ldpr, const double* Vr, int64_t ldvr, int nonneg, int col0, int ncols,
                 double* out, int64_t ldo, double* part, cudaStream_t st);
 // The same pass from exact 8-bit digits of the factors on the tensor cores
 // (cr_post_tc.cu).  Digits of an n x K factor: post_tc_digit_elems 16-bit words,
-// and n scales; *odd is set where a factor cannot be scaled, and the pass then
-// leaves empty statistics.  post_tc_blocks() = 0: not available.
+// and n scales; *odd is set where a factor cannot be scaled.  wide (post_wide_tiles
+// bytes): set to 1 for the tiles that post_tiles has to take, whose entries the digits
+// would not hold to a float64 sum's accuracy.  post_tc_blocks() = 0: not available.
 int post_tc_blocks();
 int post_tc_parts(int ny, int ncols);
 size_t post_tc_digit_elems(int n, int K);
 void post_tc_digits(int n, int K, const double* A, int64_t lda, void* digits, double* scale, int* odd, cudaStream_t st);
-void post_tc_tiles(const int* odd, int ny, int nx, int j, const void* P, const double* sP, const void* V,
+size_t post_wide_tiles(int ny, int ncols);
+void post_tc_tiles(const int* odd, uint8_t* wide, int ny, int nx, int j, const void* P, const double* sP, const void* V,
                    const double* sV, int jr, const void* Pr, const double* sPr, const void* Vr, const double* sVr,
                    int nonneg, int col0, int ncols, double* out, int64_t ldo, double* part, cudaStream_t st);
 // out[0..PS_N) = the fixed-order combination of nparts rows of statistics

@@ -1,5 +1,5 @@
 // Post-processing of a greedy solution W = U Z V^T: one tiled float64 pass (the
-// form for small ranks and for factors that cr_post_tc.cu cannot scale)
+// form for small ranks, and for the tiles that cr_post_tc.cu's digits do not hold)
 // that forms W on chip (64 x 64 tiles, never the whole ny x nx matrix),
 // optionally projects it onto the nonnegative orthant (Sec. 4, dropping the
 // nonnegativity constraint), compares it with a reference W* = U* Z* V*^T
@@ -58,8 +58,8 @@ __device__ __forceinline__ void tile_product(int nrow, int ncol, int K, const do
 // Tile t (row-tile fastest) belongs to CTA t mod gridDim.x.  out (may be null)
 // receives P(W) for the columns of this launch, column c at out + (c - col0) * ldo.
 // part[blockIdx.x * PS_N + q] receives the CTA's statistics.
-// run_if (may be null): the pass runs only where *run_if is set, else it leaves empty statistics.
-__global__ void __launch_bounds__(PTHREADS) post_tile_kernel(const int* __restrict__ run_if, int ny, int j, const double* __restrict__ P,
+// only (may be null): the tiles to take, one byte each; the others add nothing to the statistics.
+__global__ void __launch_bounds__(PTHREADS) post_tile_kernel(const uint8_t* __restrict__ only, int ny, int j, const double* __restrict__ P,
                                                              int64_t ldp, const double* __restrict__ V, int64_t ldv,
                                                              int jr, const double* __restrict__ Pr, int64_t ldpr,
                                                              const double* __restrict__ Vr, int64_t ldvr, int nonneg,
@@ -74,8 +74,8 @@ __global__ void __launch_bounds__(PTHREADS) post_tile_kernel(const int* __restri
   double s[PS_N];
 #pragma unroll
   for (int q = 0; q < PS_N; ++q) s[q] = stat_identity(q);
-  const int64_t nrun = run_if && !*run_if ? 0 : ntiles;
-  for (int64_t t = blockIdx.x; t < nrun; t += gridDim.x) {
+  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    if (only && !only[t]) continue;
     const int i0 = (int)(t % rt) * PT, c0 = col0 + (int)(t / rt) * PT;
     double acc[4][4], accr[4][4];
 #pragma unroll
@@ -130,12 +130,12 @@ int post_tiles_parts(int ny, int ncols) {
   return (int)std::min<int64_t>(post_blocks(), std::max<int64_t>(ntiles, 1));
 }
 
-void post_tiles(const int* run_if, int ny, int j, const double* P, int64_t ldp, const double* V, int64_t ldv, int jr,
+void post_tiles(const uint8_t* only, int ny, int j, const double* P, int64_t ldp, const double* V, int64_t ldv, int jr,
                 const double* Pr, int64_t ldpr, const double* Vr, int64_t ldvr, int nonneg, int col0, int ncols,
                 double* out, int64_t ldo, double* part, cudaStream_t st) {
   const int nb = post_tiles_parts(ny, ncols);
   count_launch();
-  post_tile_kernel<<<nb, PTHREADS, 0, st>>>(run_if, ny, j, P, ldp, V, ldv, jr, Pr, ldpr, Vr, ldvr, nonneg, col0, ncols,
+  post_tile_kernel<<<nb, PTHREADS, 0, st>>>(only, ny, j, P, ldp, V, ldv, jr, Pr, ldpr, Vr, ldvr, nonneg, col0, ncols,
                                             out, ldo, part);
 }
 

@@ -10,12 +10,20 @@
 //   W(i, c) = 2^(eP_i + eV_c - 14) sum_l 2^(-8 l) L_l,  L_l = sum_{s + t = l} sum_k p_s v_t.
 // Every product is an integer of at most 2^14 and every partial sum of a level over
 // at most 112 columns stays below 2^24, so bfloat16 matrix instructions with float32
-// accumulation form L_0 .. L_7 without a rounding error.  Levels 8 and up are
-// dropped: below 7 K 2^-64 of the two rows' largest entries' product, under the
-// rounding of a float64 sum.  Two 48-bit integers hold the eight levels; one float64
-// FMA and one scaled addition per 112 columns turn them into W.
-// Measured (7,530^2 entries, ms per report): rank 100 against rank 140 25.2 -> 5.4,
-// rank 100 alone 11.5 -> 2.3, rank 1 2.6 -> 1.5 (what the statistics' float64
+// accumulation form L_0 .. L_7 without a rounding error.  Two 48-bit integers hold
+// the eight levels; one float64 FMA and one scaled addition per 112 columns turn them
+// into W.
+// What is left out, levels 8 and up (seven products of at most 2^14 2^-64 a column and
+// less behind them) and the factors' digits 9 and up, is below E = 9.1 K 2^-50 in units
+// of 2^(eP_i + eV_c - 14).  A float64 sum rounds by K 2^-53 S, S = sum_k |P(i, k)| |V(c, k)|
+// in the same units, however much smaller than the rows' largest entries S is.  So
+// post_check_kernel first forms T = sum_k |p_0| |v_0|, one matrix product of the 36: a
+// digit that is not zero is at most twice its entry, hence S >= T / 4, and T >= 512
+// makes E at most 0.57 of the float64 sum's bound.  Tiles of 64 x 64 entries in which
+// some T is smaller (rows whose large entries do not meet, and the sign and size of W
+// there) go to the float64 pass, the others come from the digits.
+// Measured (7,530^2 entries, ms per report): rank 100 against rank 140 25.2 -> 5.8 (0.4 of
+// them the check), before the check rank 100 alone 11.5 -> 2.3, rank 1 2.6 -> 1.5 (what the statistics' float64
 // operations take); W's error against extended precision 6.6e-16 -> 3.9e-16 at rank
 // 140.  A warp holds 16 x 16 entries (eight levels: 64 accumulators), eight warps a
 // CTA and two CTAs an SM; W and the statistics wait in shared memory meanwhile (kept
@@ -50,7 +58,7 @@ __device__ __forceinline__ int pow2_above(double m) {
 }
 
 // Digits of the rows of A (n x K, A(r, k) at A[r + k lda]): plane s of row r at
-// out + (s * n + r) * Kp (k contiguous, zero-padded to Kp), scale[r] = 2^(e_r - 35).
+// out + (s * n + r) * Kp (k contiguous, zero-padded to Kp), scale[r] = 2^(e_r - 35) (0: a row of zeros).
 // One thread per row and group of eight columns.  *odd is set where a row holds a
 // value that is not finite or is too large or small to scale (the caller's float64
 // pass then runs instead).
@@ -76,7 +84,7 @@ __global__ void __launch_bounds__(256) post_digits_kernel(int n, int K, int Kp, 
   const int e = m > 0.0 && !bad ? pow2_above(m) : 0;
   if (r >= n) return;
   if (w == 0) {
-    scale[r] = ldexp(1.0, e - 35);
+    scale[r] = m > 0.0 ? ldexp(1.0, e - 35) : 0.0;
     if (bad) *odd = 1;
   }
   const double up = ldexp(1.0, 7 - e);
@@ -119,6 +127,58 @@ struct DigitMat {
   const double* scale;
   int n, Kp;
 };
+
+// Whether T = sum_k |p_0| |v_0| reaches 512 in the thread's entries of the 64 x 64 tile at (i0, c0),
+// rows past the matrix and rows of zeros aside: eight warps of 16 x 32 entries, the operands
+// read from global memory as the matrix instruction's fragments hold them.
+__device__ __forceinline__ bool tile_covered(const DigitMat& P, const DigitMat& V, int K, int i0, int c0, int ny, int cend) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
+  const int i = i0 + (wid & 3) * 16 + g, c = c0 + (wid >> 2) * 32;
+  auto word = [&](const DigitMat& M, int row, int end, int k) -> uint32_t {  // two digits' sizes
+    return row < end ? __ldg(reinterpret_cast<const uint32_t*>(M.d + (int64_t)row * M.Kp + k)) & 0x7FFF7FFFu : 0u;
+  };
+  float acc[4][4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[t][u] = 0.f;
+  __syncwarp();
+  for (int k = 0; k < K; k += 16) {
+    const uint32_t a[4] = {word(P, i, ny, k + 2 * q), word(P, i + 8, ny, k + 2 * q), word(P, i, ny, k + 2 * q + 8),
+                           word(P, i + 8, ny, k + 2 * q + 8)};
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      mma16816(acc[t], a, word(V, c + 8 * t + g, cend, k + 2 * q), word(V, c + 8 * t + g, cend, k + 2 * q + 8));
+  }
+  bool ok = true;
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int ii = i + 8 * (u >> 1), cc = c + 8 * t + 2 * q + (u & 1);
+      if (ii < ny && cc < cend && acc[t][u] < 512.f) ok = ok && (P.scale[ii] == 0.0 || V.scale[cc] == 0.0);
+    }
+  return ok;
+}
+
+// wide[t] = 1 for the 64 x 64 tiles t (row tile fastest) that the float64 pass has to take
+__global__ void __launch_bounds__(kPcThreads) post_check_kernel(const int* __restrict__ odd, int ny, int j, DigitMat P,
+                                                                DigitMat V, int jr, DigitMat Pr, DigitMat Vr, int col0,
+                                                                int ncols, uint8_t* __restrict__ wide) {
+  const int rt = (ny + 63) / 64, cend = col0 + ncols;
+  const int64_t ntiles = (int64_t)rt * ((ncols + 63) / 64);
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int i0 = (int)(tile % rt) * 64, c0 = col0 + (int)(tile / rt) * 64;
+    bool ok = !*odd;  // the same in all threads, as is jr: the matrix instructions take whole warps
+    if (ok) {
+      ok = tile_covered(P, V, j, i0, c0, ny, cend);
+      const bool ref = jr == 0 || tile_covered(Pr, Vr, jr, i0, c0, ny, cend);
+      ok = ok && ref;
+    }
+    const int bad = __syncthreads_or(!ok);
+    if (threadIdx.x == 0) wide[tile] = bad ? 1 : 0;
+  }
+}
 
 // byte offset of 16-byte piece q of a staged row: the pieces of every second group of four rows are
 // swapped, which puts those of eight consecutive rows in distinct banks
@@ -274,9 +334,9 @@ struct TcStats {
 };
 
 // As post_tile_kernel (cr_post.cu), on the digit planes of P, V and the reference's
-// factors; leaves empty statistics where *odd is set.
-__global__ void __launch_bounds__(kPcThreads, 2) post_tc_kernel(const int* __restrict__ odd, int ny, int j, DigitMat P, DigitMat V,
-                                                           int jr, DigitMat Pr, DigitMat Vr, int nonneg, int col0,
+// factors; passes the tiles by that post_check_kernel marked.
+__global__ void __launch_bounds__(kPcThreads, 2) post_tc_kernel(const uint8_t* __restrict__ wide, int ny, int j, DigitMat P,
+                                                           DigitMat V, int jr, DigitMat Pr, DigitMat Vr, int nonneg, int col0,
                                                            int ncols, double* __restrict__ out, int64_t ldo,
                                                            double* __restrict__ part) {
   extern __shared__ __align__(16) char buf[];  // see kSmem
@@ -286,12 +346,13 @@ __global__ void __launch_bounds__(kPcThreads, 2) post_tc_kernel(const int* __res
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, wr = wid & 3, wc = wid >> 2;
   const int g = lane >> 2, cb = 2 * (lane & 3);
   const int rt = (ny + kTm - 1) / kTm, ct = (ncols + kTn - 1) / kTn;
-  const int64_t ntiles = *odd ? 0 : (int64_t)rt * ct;
+  const int64_t ntiles = (int64_t)rt * ct;
   const int cend = col0 + ncols;
   TcStats ts;
   ts.save(st);
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int i0 = (int)(tile % rt) * kTm, c0 = col0 + (int)(tile / rt) * kTn;
+    if (wide[tile % rt + tile / rt / 2 * rt]) continue;  // its half of a 64 x 64 tile
     if (jr > 0) tile_product(buf, Pr, Vr, jr, i0, c0, rt_);
     tile_product(buf, P, V, j, i0, c0, wt);
     ts.load(st);
@@ -352,16 +413,21 @@ void post_tc_digits(int n, int K, const double* A, int64_t lda, void* digits, do
   post_digits_kernel<<<(n + 31) / 32, 256, 0, st>>>(n, K, padded(K), A, lda, (__nv_bfloat16*)digits, scale, odd);
 }
 
-void post_tc_tiles(const int* odd, int ny, int nx, int j, const void* P, const double* sP, const void* V, const double* sV,
-                   int jr, const void* Pr, const double* sPr, const void* Vr, const double* sVr, int nonneg, int col0,
-                   int ncols, double* out, int64_t ldo, double* part, cudaStream_t st) {
+size_t post_wide_tiles(int ny, int ncols) { return (size_t)((ny + 63) / 64) * ((ncols + 63) / 64); }
+
+void post_tc_tiles(const int* odd, uint8_t* wide, int ny, int nx, int j, const void* P, const double* sP, const void* V,
+                   const double* sV, int jr, const void* Pr, const double* sPr, const void* Vr, const double* sVr,
+                   int nonneg, int col0, int ncols, double* out, int64_t ldo, double* part, cudaStream_t st) {
   auto mat = [&](const void* d, const double* s, int n, int K) {
     return DigitMat{(const __nv_bfloat16*)d, s, n, padded(K)};
   };
+  const DigitMat mP = mat(P, sP, ny, j), mV = mat(V, sV, nx, j), mPr = mat(Pr, sPr, ny, jr), mVr = mat(Vr, sVr, nx, jr);
   count_launch();
-  post_tc_kernel<<<post_tc_parts(ny, ncols), kPcThreads, kSmem, st>>>(
-      odd, ny, j, mat(P, sP, ny, j), mat(V, sV, nx, j), jr, mat(Pr, sPr, ny, jr), mat(Vr, sVr, nx, jr), nonneg, col0,
-      ncols, out, ldo, part);
+  post_check_kernel<<<(unsigned)std::min<size_t>(post_wide_tiles(ny, ncols), 1 << 16), kPcThreads, 0, st>>>(
+      odd, ny, j, mP, mV, jr, mPr, mVr, col0, ncols, wide);
+  count_launch();
+  post_tc_kernel<<<post_tc_parts(ny, ncols), kPcThreads, kSmem, st>>>(wide, ny, j, mP, mV, jr, mPr, mVr, nonneg, col0,
+                                                                      ncols, out, ldo, part);
 }
 
 }  // namespace cr
