@@ -1590,10 +1590,11 @@ cr_status grow_projections(cr_problem* p, int q) {
     b.row[g][2] = m2[g] + q;
   }
   b.ldrow = ld;
+  b.mag = p->bcoef + 2 * ld;
   panel_t(b, st);
   spmv_xt(m, p->xc_ptr, p->xc_row, p->xc_val, vq, p->H + q, ld, st);
   gemv_t(ny, m, p->OmY, ny, uq, p->P + q, ld, 1.0, 0.0, st);
-  omega_border(q, m, p->UU, ldu, p->bcoef, p->om_ptr, p->om_row, p->om_full, p->G, ld, st);
+  omega_border(q, m, p->UU, ldu, p->bcoef, b.mag, p->om_ptr, p->om_row, p->om_full, p->Om, ny, p->G, ld, st);
   return grow_bases(p, q);
 }
 

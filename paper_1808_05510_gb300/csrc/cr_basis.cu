@@ -31,17 +31,19 @@ __device__ __forceinline__ double wsum(double v) {
 }
 
 // out[p + s * ldo] = A(:, p)^T w_s, s < 3 (column s at at[s] if given, and mirrored into a row with
-// stride ldrow if given); one CTA per column p and grid, fixed-order sums
+// stride ldrow if given); one CTA per column p and grid, fixed-order sums.
+// MAG: grid 0 also gives mag[p] = sum_i |A(i, p)| |w_0(i)|
+template <bool MAG>
 __global__ void __launch_bounds__(256) panel_t_kernel(const PanelArgs a) {
   const int g = blockIdx.y, p = blockIdx.x, n = a.n[g];
   if (p >= a.k[g]) return;
   const double* A = a.A[g] + (int64_t)p * a.lda[g];
   const double* w = a.w[g];
   const int64_t ldw = a.ldw[g];
-  constexpr int NV = 3;
-  double acc[NV][2];
+  constexpr int NV = 3, NS = MAG ? NV + 1 : NV;
+  double acc[NS][2];
 #pragma unroll
-  for (int s = 0; s < NV; ++s) acc[s][0] = acc[s][1] = 0.0;
+  for (int s = 0; s < NS; ++s) acc[s][0] = acc[s][1] = 0.0;
   int i = threadIdx.x;
   for (; i + 256 < n; i += 512) {
     const double x0 = A[i], x1 = A[i + 256];
@@ -50,25 +52,32 @@ __global__ void __launch_bounds__(256) panel_t_kernel(const PanelArgs a) {
       acc[s][0] = fma(x0, w[i + s * ldw], acc[s][0]);
       acc[s][1] = fma(x1, w[i + 256 + s * ldw], acc[s][1]);
     }
+    if (MAG && g == 0) {
+      acc[NS - 1][0] = fma(fabs(x0), fabs(w[i]), acc[NS - 1][0]);
+      acc[NS - 1][1] = fma(fabs(x1), fabs(w[i + 256]), acc[NS - 1][1]);
+    }
   }
   if (i < n) {
     const double x0 = A[i];
 #pragma unroll
     for (int s = 0; s < NV; ++s) acc[s][0] = fma(x0, w[i + s * ldw], acc[s][0]);
+    if (MAG && g == 0) acc[NS - 1][0] = fma(fabs(x0), fabs(w[i]), acc[NS - 1][0]);
   }
   // one warp per value adds the 256 partial sums (a shuffle tree in every warp costs three times
   // the float64 issue slots)
-  __shared__ double sh[NV][256];
+  __shared__ double sh[NS][256];
 #pragma unroll
-  for (int s = 0; s < NV; ++s) sh[s][threadIdx.x] = acc[s][0] + acc[s][1];
+  for (int s = 0; s < NS; ++s) sh[s][threadIdx.x] = acc[s][0] + acc[s][1];
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (wid < NV) {
+  if (wid < NS) {
     double q[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) q[u] = sh[wid][lane + 32 * u];
     const double t = wsum(((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7])));
-    if (lane == 0) {
+    if (MAG && wid == NV) {
+      if (lane == 0 && g == 0) a.mag[p] = t;
+    } else if (lane == 0) {
       (a.at[g][wid] ? a.at[g][wid] : a.out[g] + wid * a.ldo[g])[p] = t;
       if (a.row[g][wid]) a.row[g][wid][(int64_t)p * a.ldrow] = t;
     }
@@ -278,25 +287,39 @@ __global__ void __launch_bounds__(256) basis_product_kernel(int n1, int64_t ld, 
 // injection's row lists: the unobserved rows (full[a] = 1: D minus their products) or the observed
 // ones; one warp per (p, a), both triangles written.  The shorter list needs at most half of the
 // products of a masked copy of u_q times U (gemm: 20.7 of 141 ms at rank 240, 28 injections), and
-// bounds the launch by its gathers from L2.
+// bounds the launch by its gathers from L2.  The difference carries the rounding of all rows'
+// products: it is taken where the unobserved rows hold at most half of T(p) = sum_i |u_p(i)| |u_q(i)|,
+// which keeps its error within three times the observed rows' own; elsewhere the sum runs over the
+// observed rows themselves.
 __global__ void __launch_bounds__(256) omega_border_kernel(int q, int m, const double* __restrict__ UU, int64_t ldu,
-                                                           const double* __restrict__ D, const int* __restrict__ zp,
-                                                           const int* __restrict__ zrow, const uint8_t* __restrict__ full,
-                                                           double* __restrict__ G, int64_t ld) {
+                                                           const double* __restrict__ D, const double* __restrict__ T,
+                                                           const int* __restrict__ zp, const int* __restrict__ zrow,
+                                                           const uint8_t* __restrict__ full, const uint8_t* __restrict__ Om,
+                                                           int n, double* __restrict__ G, int64_t ld) {
   const int lane = threadIdx.x & 31;
   const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (t >= (int64_t)m * (q + 1)) return;
   const int p = (int)(t % (q + 1)), a = (int)(t / (q + 1));
   const double *up = UU + p * ldu, *uq = UU + q * ldu;
-  double acc = 0.0;
+  double acc = 0.0, mag = 0.0;
 #pragma unroll 4
   for (int k = zp[a] + lane; k < zp[a + 1]; k += 32) {
     const int i = zrow[k];
     acc = fma(up[i], uq[i], acc);
+    mag = fma(fabs(up[i]), fabs(uq[i]), mag);
   }
   acc = wsum(acc);
+  double g = acc;
+  if (full[a]) {
+    g = D[p] - acc;
+    if (!(2.0 * wsum(mag) <= T[p])) {
+      acc = 0.0;
+      for (int i = lane; i < n; i += 32)
+        if (Om[i + (int64_t)a * n]) acc = fma(up[i], uq[i], acc);
+      g = wsum(acc);
+    }
+  }
   if (lane == 0) {
-    const double g = full[a] ? D[p] - acc : acc;
     double* Ga = G + (int64_t)a * ld * ld;
     Ga[p + (int64_t)q * ld] = g;
     Ga[q + (int64_t)p * ld] = g;
@@ -305,19 +328,22 @@ __global__ void __launch_bounds__(256) omega_border_kernel(int q, int m, const d
 
 }  // namespace
 
-void omega_border(int q, int m, const double* UU, int64_t ldu, const double* D, const int* zp, const int* zrow,
-                  const uint8_t* full, double* G, int64_t ld, cudaStream_t st) {
+void omega_border(int q, int m, const double* UU, int64_t ldu, const double* D, const double* T, const int* zp,
+                  const int* zrow, const uint8_t* full, const uint8_t* Om, int n, double* G, int64_t ld, cudaStream_t st) {
   const int64_t t = (int64_t)m * (q + 1);
   if (t <= 0) return;
   count_launch();
-  omega_border_kernel<<<(unsigned)((t + 7) / 8), 256, 0, st>>>(q, m, UU, ldu, D, zp, zrow, full, G, ld);
+  omega_border_kernel<<<(unsigned)((t + 7) / 8), 256, 0, st>>>(q, m, UU, ldu, D, T, zp, zrow, full, Om, n, G, ld);
 }
 
 void panel_t(const PanelArgs& a, cudaStream_t st) {
   const int k = std::max(a.k[0], a.k[1]);
   if (k <= 0) return;
   count_launch();
-  panel_t_kernel<<<dim3(k, 2), 256, 0, st>>>(a);
+  if (a.mag)
+    panel_t_kernel<true><<<dim3(k, 2), 256, 0, st>>>(a);
+  else
+    panel_t_kernel<false><<<dim3(k, 2), 256, 0, st>>>(a);
 }
 
 void panel_n(const PanelArgs& a, cudaStream_t st) {

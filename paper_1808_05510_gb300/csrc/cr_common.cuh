@@ -440,13 +440,15 @@ struct PanelArgs {
   const double* src[2] = {nullptr, nullptr};  // the three source columns, leading dimension lds
   int64_t lds[2] = {0, 0};
   double* count[2] = {nullptr, nullptr};
+  double* mag = nullptr;  // grid 0, panel_t: sum_i |A(i, p)| |w_0(i)| (null: not formed)
 };
 // out(p, s) = A(:, p)^T w_s, three columns
 void panel_t(const PanelArgs& a, cudaStream_t st);
-// Column and row q of every G_a = U^T diag(Omega_a) U (u_p at UU + p ldu), from D(p) = u_p^T u_q and
-// row lists: the unobserved rows of injection a (full[a]) or its observed ones
-void omega_border(int q, int m, const double* UU, int64_t ldu, const double* D, const int* zp, const int* zrow,
-                  const uint8_t* full, double* G, int64_t ld, cudaStream_t st);
+// Column and row q of every G_a = U^T diag(Omega_a) U (u_p at UU + p ldu), from D(p) = u_p^T u_q,
+// T(p) = |u_p|^T |u_q| and row lists: the unobserved rows of injection a (full[a]) or its observed
+// ones.  Om: n x m, contiguous
+void omega_border(int q, int m, const double* UU, int64_t ldu, const double* D, const double* T, const int* zp,
+                  const int* zrow, const uint8_t* full, const uint8_t* Om, int n, double* G, int64_t ld, cudaStream_t st);
 // w_s -= A out(:, s), three columns
 void panel_n(const PanelArgs& a, cudaStream_t st);
 // w_s = src_s, three columns
