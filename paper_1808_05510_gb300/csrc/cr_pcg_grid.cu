@@ -49,6 +49,7 @@ namespace {
 // One CTA of 1,024 threads per SM with the 16-bit table, at most two of 512 with the general one:
 // (every further CTA lengthens the barriers and the sums behind them).
 constexpr int kGThreads16 = 1024, kGThreads = 512;
+constexpr int kMaxInj = 4096;  // injections of a problem
 
 struct GridPcg {
   DevLap L;
@@ -128,22 +129,22 @@ __device__ __forceinline__ void st4(double* p, const double (&v)[4]) {
   *reinterpret_cast<double2*>(p + 2) = double2{v[2], v[3]};
 }
 
-// Block sums of NV accumulators in a fixed tree order; results in out[] of thread 0.
+// Block sums of NV accumulators in a fixed tree order; results in out[] of thread 0.  sh: NV blockDim
+// doubles of the kernel's one buffer (a static array in each instantiation came to 49,696 B).
 // Float64 adds take 16 issue cycles a warp, so a shuffle tree over every warp costs
 // 2,560 of them per value at 1,024 threads: the double-float form sums its warps in
 // float32, the float64 form lets 128 threads add eight values each from shared memory.
 template <int NV>
-__device__ __forceinline__ void block_reduce(Acc<float> (&v)[NV], double* out) {
-  __shared__ double sh[32][NV];
+__device__ __forceinline__ void block_reduce(Acc<float> (&v)[NV], double* sh, double* out) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     const DF t = warp_sum_df(v[k].v);
-    if (lane == 0) sh[w][k] = (double)t.hi + (double)t.lo;
+    if (lane == 0) sh[w * NV + k] = (double)t.hi + (double)t.lo;
   }
   __syncthreads();
   if (w < NV) {
-    double t = lane < nw ? sh[lane][w] : 0.0;
+    double t = lane < nw ? sh[lane * NV + w] : 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
     if (lane == 0) out[w] = t;
@@ -151,18 +152,18 @@ __device__ __forceinline__ void block_reduce(Acc<float> (&v)[NV], double* out) {
   __syncthreads();
 }
 template <int NV>
-__device__ __forceinline__ void block_reduce(Acc<double> (&v)[NV], double* out) {
-  __shared__ double sh[NV][kGThreads16], sw[4][NV];
+__device__ __forceinline__ void block_reduce(Acc<double> (&v)[NV], double* sh, double* out) {
+  __shared__ double sw[4][NV];
   const int nt = blockDim.x;  // 512 or 1,024
 #pragma unroll
-  for (int k = 0; k < NV; ++k) sh[k][threadIdx.x] = v[k].v;
+  for (int k = 0; k < NV; ++k) sh[k * nt + threadIdx.x] = v[k].v;
   __syncthreads();
   if (threadIdx.x < 128) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
       double q[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) q[u] = threadIdx.x + 128 * u < nt ? sh[k][threadIdx.x + 128 * u] : 0.0;
+      for (int u = 0; u < 8; ++u) q[u] = threadIdx.x + 128 * u < nt ? sh[k * nt + threadIdx.x + 128 * u] : 0.0;
       double t = ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
@@ -336,7 +337,7 @@ __device__ __forceinline__ T data_row(const GridPcg& a, const T* om, const doubl
 template <class T, int KM, bool F16>
 __global__ void __launch_bounds__(F16 ? kGThreads16 : kGThreads, 1) pcg_grid_kernel(const GridPcg a) {
   extern __shared__ double ys[];  // v side: y = s o (X^T v), m entries
-  __shared__ double red[kParts];
+  __shared__ double red[kParts], sums[3 * (F16 ? kGThreads16 : kGThreads)];
   T* xs = (T*)a.xs;
   T* rs = (T*)a.rs;
   T* qs = (T*)a.qs;
@@ -390,7 +391,7 @@ __global__ void __launch_bounds__(F16 ? kGThreads16 : kGThreads, 1) pcg_grid_ker
       acc[1].add(ri, ri);
       acc[2].add(bi, bi);
     });
-    block_reduce(acc, red);
+    block_reduce(acc, sums, red);
     if (threadIdx.x == 0) {
       double* pb = a.part + (size_t)blockIdx.x * kParts;
       pb[1] = red[0];
@@ -449,7 +450,7 @@ __global__ void __launch_bounds__(F16 ? kGThreads16 : kGThreads, 1) pcg_grid_ker
           qs[i] = qi;
           acc[0].add(pi, qi);
         });
-        block_reduce(acc, red);
+        block_reduce(acc, sums, red);
         if (threadIdx.x == 0) a.part[(size_t)blockIdx.x * kParts + 0] = red[0];
       }
       if (!grid_bar_sync(bar)) goto done;
@@ -486,7 +487,7 @@ __global__ void __launch_bounds__(F16 ? kGThreads16 : kGThreads, 1) pcg_grid_ker
           st4(rs + i, rv);
           st4(zs + i, zv);
         }
-        block_reduce(acc, red);
+        block_reduce(acc, sums, red);
         if (threadIdx.x == 0) {
           double* pb = a.part + (size_t)blockIdx.x * kParts;
           pb[1] = red[0];
@@ -536,8 +537,10 @@ int pcg_grid_blocks(bool fp32, int m, const DevLap& L) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const size_t smem = sizeof(double) * (size_t)std::max(m, 1);
-  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, grid_kernel_fn(fp32, L), grid_threads(L), smem);
-  if (e != cudaSuccess || per < 1) {
+  const void* fn = grid_kernel_fn(fp32, L);
+  // y and the sums together may exceed the 48 KB that need no opt-in (m up to 4,096: 32 KB + 25 KB)
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(double) * kMaxInj) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, grid_threads(L), smem) != cudaSuccess || per < 1) {
     cudaGetLastError();
     return 0;
   }
