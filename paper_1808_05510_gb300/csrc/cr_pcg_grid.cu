@@ -22,7 +22,7 @@
 // Every block adds the per-block partial sums itself, in one fixed order, so
 // all blocks hold bit-identical scalars and take identical decisions.
 // T = float: float32 vectors and arithmetic with double-float (two-float)
-// accumulation of the inner products; T = double: float64 throughout (on
+// accumulation of the inner products per thread, float64 between threads; T = double: float64 throughout (on
 // GB300 the float64 form is bound by float64 arithmetic, not by HBM).
 // Neighbour tables: a unit-weight graph Laplacian with at most six neighbours
 // per row, none further than 32,767 rows away, stores the six distances as
@@ -99,11 +99,13 @@ template <>
 struct Acc<float> {
   DF v{0.f, 0.f};
   __device__ void add(float a, float b) { v = df_add(v, df_prod(a, b)); }
+  __device__ double get() const { return (double)v.hi + (double)v.lo; }
 };
 template <>
 struct Acc<double> {
   double v = 0.0;
   __device__ void add(double a, double b) { v = fma(a, b, v); }
+  __device__ double get() const { return v; }
 };
 
 // four consecutive rows of a vector
@@ -129,34 +131,16 @@ __device__ __forceinline__ void st4(double* p, const double (&v)[4]) {
   *reinterpret_cast<double2*>(p + 2) = double2{v[2], v[3]};
 }
 
-// Block sums of NV accumulators in a fixed tree order; results in out[] of thread 0.  sh: NV blockDim
-// doubles of the kernel's one buffer (a static array in each instantiation came to 49,696 B).
-// Float64 adds take 16 issue cycles a warp, so a shuffle tree over every warp costs
-// 2,560 of them per value at 1,024 threads: the double-float form sums its warps in
-// float32, the float64 form lets 128 threads add eight values each from shared memory.
-template <int NV>
-__device__ __forceinline__ void block_reduce(Acc<float> (&v)[NV], double* sh, double* out) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    const DF t = warp_sum_df(v[k].v);
-    if (lane == 0) sh[w * NV + k] = (double)t.hi + (double)t.lo;
-  }
-  __syncthreads();
-  if (w < NV) {
-    double t = lane < nw ? sh[lane * NV + w] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) out[w] = t;
-  }
-  __syncthreads();
-}
-template <int NV>
-__device__ __forceinline__ void block_reduce(Acc<double> (&v)[NV], double* sh, double* out) {
+// Block sums of NV accumulators in float64 and a fixed tree order; results in out[] of thread 0.
+// Float64 adds take 16 issue cycles a warp, so a shuffle tree over every warp costs 2,560 of them per
+// value at 1,024 threads: instead 128 threads add eight values each from shared memory.  sh: NV
+// blockDim doubles of the kernel's one buffer (a static array in each instantiation came to 49,696 B).
+template <class T, int NV>
+__device__ __forceinline__ void block_reduce(Acc<T> (&v)[NV], double* sh, double* out) {
   __shared__ double sw[4][NV];
   const int nt = blockDim.x;  // 512 or 1,024
 #pragma unroll
-  for (int k = 0; k < NV; ++k) sh[k * nt + threadIdx.x] = v[k].v;
+  for (int k = 0; k < NV; ++k) sh[k * nt + threadIdx.x] = v[k].get();
   __syncthreads();
   if (threadIdx.x < 128) {
 #pragma unroll
