@@ -161,7 +161,9 @@ typedef struct {
   uint64_t seed;           /* seed of the fallback ALS start vector */
   void* stream;            /* cudaStream_t for all device work; NULL = a library-owned stream */
   /* Optional device allocator (e.g. a framework caching allocator).  When
-   * alloc is NULL the library uses cudaMalloc/cudaFree. */
+   * alloc is NULL the library uses cudaMalloc/cudaFree.  A block that does not
+   * start at a multiple of 256 bytes is given back and asked for again, 256
+   * bytes larger. */
   void* (*alloc)(size_t bytes, void* ctx);
   void (*free)(void* ptr, size_t bytes, void* ctx);
   void* alloc_ctx;

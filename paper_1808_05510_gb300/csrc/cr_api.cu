@@ -178,7 +178,7 @@ struct cr_problem {
   bool own_stream = false;
   std::string err;
   int j = 0;
-  std::vector<std::pair<void*, size_t>> allocs;
+  std::vector<std::pair<void*, size_t>> allocs;  // as the allocator gave them
   DevLap Lx, Ly;
   DevMg mg[2];  // multigrid hierarchies of L_y (side 0) and L_x (side 1)
   DevPush push[2];  // float32 cluster PCG of the u side (L_y) and the v side (L_x)
@@ -356,12 +356,21 @@ cr_status fail(cr_problem* p, cr_status s, const std::string& msg) {
   return s;
 }
 
+// Buffers start at multiples of 256 bytes, as cudaMalloc's do: 16-byte loads, asynchronous copies and
+// tensor maps rely on it.  A caller's allocator that returns others is asked for as much more.
+constexpr size_t kAlign = 256;
+
 template <class T>
 cr_status dalloc(cr_problem* p, T** out, size_t count) {
-  const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
+  size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
   void* ptr = nullptr;
   if (p->opt.alloc) {
     ptr = p->opt.alloc(bytes, p->opt.alloc_ctx);
+    if (ptr && reinterpret_cast<uintptr_t>(ptr) % kAlign) {
+      p->opt.free(ptr, bytes, p->opt.alloc_ctx);
+      bytes += kAlign;
+      ptr = p->opt.alloc(bytes, p->opt.alloc_ctx);
+    }
     if (!ptr) return fail(p, CR_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes failed");
   } else {
     cudaError_t e = cudaMalloc(&ptr, bytes);
@@ -371,7 +380,7 @@ cr_status dalloc(cr_problem* p, T** out, size_t count) {
     }
   }
   p->allocs.push_back({ptr, bytes});
-  *out = static_cast<T*>(ptr);
+  *out = reinterpret_cast<T*>((reinterpret_cast<uintptr_t>(ptr) + kAlign - 1) / kAlign * kAlign);
   CUCHK(p, cudaMemsetAsync(ptr, 0, bytes, p->st));
   return CR_OK;
 }
