@@ -3145,26 +3145,40 @@ cr_status cr_solution_report(cr_problem* p, int32_t nonneg, int32_t jr, const do
   }
   // tensor-core form: digits of the four factors, and the float64 pass behind it for
   // the tiles that they do not hold
-  const bool tc = j > 0 && (j + jr >= kPostTcRank || out->entries >= kPostTcEntries) && post_tc_blocks() > 0;
+  bool tc = j > 0 && (j + jr >= kPostTcRank || out->entries >= kPostTcEntries) && post_tc_blocks() > 0;
+  auto dig_rows = [&](int k) { return k % 2 == 0 ? ny : nx; };  // P, V, Pr, Vr
+  auto dig_rank = [&](int k) { return k < 2 ? j : jr; };
   if (tc) {
-    if (!p->post_odd) TRY(dalloc(p, &p->post_odd, 1));
-    if ((int64_t)post_wide_tiles(ny, (int)cw) > p->post_wide_cap) {
-      p->post_wide_cap = (int64_t)post_wide_tiles(ny, (int)cw);
-      TRY(dalloc(p, &p->post_wide, (size_t)p->post_wide_cap));
+    auto room = [&]() -> cr_status {
+      if (!p->post_odd) TRY(dalloc(p, &p->post_odd, 1));
+      const int64_t wide = (int64_t)post_wide_tiles(ny, (int)cw);
+      if (wide > p->post_wide_cap) {
+        TRY(dalloc(p, &p->post_wide, (size_t)wide));
+        p->post_wide_cap = wide;
+      }
+      for (int k = 0; k < 4; ++k) {
+        const int cap = k < 2 ? p->rcap : p->post_ref_cap;
+        if (dig_rank(k) <= p->post_dig_cap[k]) continue;
+        if (!p->post_scale[k]) TRY(dalloc(p, &p->post_scale[k], (size_t)dig_rows(k)));
+        TRY(dalloc(p, &p->post_dig[k], post_tc_digit_elems(dig_rows(k), cap)));
+        p->post_dig_cap[k] = cap;
+      }
+      return CR_OK;
+    };
+    // the digits take twice the factors' memory: without room for them the float64 pass needs none
+    const cr_status rs = room();
+    if (rs != CR_OK && rs != CR_ENOMEM) return rs;
+    if (rs == CR_ENOMEM) {
+      tc = false;
+      p->err.clear();
     }
+  }
+  if (tc) {
     CUCHK(p, cudaMemsetAsync(p->post_odd, 0, sizeof(int), st));
     const double* src[4] = {p->post_P, p->VV, p->post_Pr, p->post_Vr};
     const int64_t lds[4] = {ny, 3 * (int64_t)nx, ny, nx};
-    for (int k = 0; k < 4; ++k) {
-      const int n = k % 2 == 0 ? ny : nx, r = k < 2 ? j : jr, cap = k < 2 ? p->rcap : p->post_ref_cap;
-      if (r == 0) continue;
-      if (r > p->post_dig_cap[k]) {
-        TRY(dalloc(p, &p->post_dig[k], post_tc_digit_elems(n, cap)));
-        if (!p->post_scale[k]) TRY(dalloc(p, &p->post_scale[k], (size_t)n));
-        p->post_dig_cap[k] = cap;
-      }
-      post_tc_digits(n, r, src[k], lds[k], p->post_dig[k], p->post_scale[k], p->post_odd, st);
-    }
+    for (int k = 0; k < 4; ++k)
+      post_tc_digits(dig_rows(k), dig_rank(k), src[k], lds[k], p->post_dig[k], p->post_scale[k], p->post_odd, st);
   }
   int64_t nparts = 0;
   for (int64_t c0 = 0; c0 < nx; c0 += cw) {
