@@ -2,8 +2,8 @@
 // box (channels 2 -> 16 -> 16 -> 16 -> 1, zero padding, ReLU between layers),
 // BF16 weights and activations, float32 accumulation, float32 gradients and
 // Adam state.  Forward, backward (data and weight) and the optimiser step are
-// hand-written kernels; reductions are fixed-order (one block per weight
-// group, then a fixed tree), so training is reproducible.
+// hand-written kernels; reductions are fixed-order (a fixed share of the rows
+// per block, blocks added in order), so training is reproducible.
 //
 // Input channels: 0 = Jacobi-scaled residual D^-1 r / s on the mask voxels,
 // 1 = the mask.  The solver uses z = D^-1 r + s * net(input) (cr_api.cu).
@@ -188,15 +188,17 @@ __global__ void __launch_bounds__(kThreads) conv_bwd_data(Dims g, int B, const A
 // between groups of threads.  One CTA per (co, ci) pair, as before, re-read every
 // input from memory for every pair and left most SMs idle on the 2 -> 16 and
 // 16 -> 1 layers: 4.55, 4.55 and 3.27 ms (8 x 40^3 voxels; loss, gradients and a
-// forward pass 19.7 ms, now 3.5).  Partial sums of the
+// forward pass 19.8 ms, now 3.2).  Partial sums of the
 // CTAs go to `part` and are added in CTA order by conv_bwd_weight_sum.
+// A row wider than XT columns (the multiple of 16 whose stage fits the 48 KB of static shared
+// memory) goes in equal pieces; 16 lanes stage a row, so that only its own columns are read.
 // A gradient of exactly zero adds nothing, and taps outside the box add nothing,
 // also beside infinities: a row that stages a non-finite value takes the checked
 // loop.
 template <int CI, int CO, class S, class A>
 __global__ void __launch_bounds__(kThreads) conv_bwd_weight(Dims g, int B, const A* __restrict__ gout,
                                                             const S* __restrict__ ain, A* __restrict__ part) {
-  constexpr int XT = sizeof(A) == 4 ? 40 : 32, XP = XT + 3, PAIRS = CI * CO, NG = kThreads / PAIRS, GP = XT + 1;
+  constexpr int XT = sizeof(A) == 4 ? 64 : 32, XP = XT + 3, PAIRS = CI * CO, NG = kThreads / PAIRS, GP = XT + 1;
   constexpr int STAGE = 9 * CI * XP + CO * GP, KC = 14, COMB = NG > 1 ? kThreads * KC : 0;
   __shared__ A sm[STAGE > COMB ? STAGE : COMB];
   A* as = sm;               // [row 0..8][ci][XP], x0 - 1 first
@@ -206,29 +208,40 @@ __global__ void __launch_bounds__(kThreads) conv_bwd_weight(Dims g, int B, const
   A acc[28];
 #pragma unroll
   for (int k = 0; k < 28; ++k) acc[k] = (A)0;
+  const int sl = threadIdx.x & 15, sg = threadIdx.x >> 4;
+  const int pieces = (g.W + XT - 1) / XT, xw = (g.W + pieces - 1) / pieces;
   const int64_t rows = (int64_t)B * g.D * g.H;
   const int64_t r0 = rows * blockIdx.x / gridDim.x, r1 = rows * (blockIdx.x + 1) / gridDim.x;
   for (int64_t r = r0; r < r1; ++r) {
     const int y = (int)(r % g.H), z = (int)((r / g.H) % g.D), b = (int)(r / ((int64_t)g.H * g.D));
-    for (int x0 = 0; x0 < g.W; x0 += XT) {
-      const int xt = min(XT, g.W - x0);
+    for (int x0 = 0; x0 < g.W; x0 += xw) {
+      const int xt = min(xw, g.W - x0);
       __syncthreads();
       int odd = 0;
-      for (int k = threadIdx.x; k < 9 * CI * XP; k += kThreads) {
-        const int xx = x0 - 1 + k % XP, c = (k / XP) % CI, q = k / (XP * CI);
-        const int zz = z + q / 3 - 1, yy = y + q % 3 - 1;
-        A v = (A)0;
-        if (xx >= 0 && xx < g.W && yy >= 0 && yy < g.H && zz >= 0 && zz < g.D)
-          v = to_acc(ain[((int64_t)b * CI + c) * g.V + ((int64_t)zz * g.H + yy) * g.W + xx]);
-        odd |= !isfinite(v);
-        as[k] = v;
+#pragma unroll 3
+      for (int k = sg; k < 9 * CI; k += kThreads / 16) {
+        const int c = k % CI, q = k / CI, zz = z + q / 3 - 1, yy = y + q % 3 - 1;
+        const bool in = yy >= 0 && yy < g.H && zz >= 0 && zz < g.D;
+        const S* src = ain + ((int64_t)b * CI + c) * g.V + ((int64_t)(in ? zz : z) * g.H + (in ? yy : y)) * g.W;
+        A v[(XT + 17) / 16];  // columns x0 - 1 .. x0 + xt
+#pragma unroll
+        for (int u = 0; u < (XT + 17) / 16; ++u) {
+          const int xx = x0 - 1 + sl + 16 * u;
+          v[u] = in && sl + 16 * u < xt + 2 && xx >= 0 && xx < g.W ? to_acc(src[xx]) : (A)0;
+        }
+#pragma unroll
+        for (int u = 0; u < (XT + 17) / 16; ++u)
+          if (sl + 16 * u < xt + 2) {
+            odd |= !isfinite(v[u]);
+            as[k * XP + sl + 16 * u] = v[u];
+          }
       }
-      for (int k = threadIdx.x; k < CO * XT; k += kThreads) {
-        const int xx = k % XT, c = k / XT;
-        const A v = xx < xt ? gout[((int64_t)b * CO + c) * g.V + ((int64_t)z * g.H + y) * g.W + x0 + xx] : (A)0;
-        odd |= !isfinite(v);
-        gs[c * GP + xx] = v;
-      }
+      for (int c = sg; c < CO; c += kThreads / 16)
+        for (int xx = sl; xx < xt; xx += 16) {
+          const A v = gout[((int64_t)b * CO + c) * g.V + ((int64_t)z * g.H + y) * g.W + x0 + xx];
+          odd |= !isfinite(v);
+          gs[c * GP + xx] = v;
+        }
       const bool checked = __syncthreads_or(odd);
       const int per = (xt + NG - 1) / NG, xa = min(xt, grp * per), xb = min(xt, xa + per);
       const A* ap = as + ci * XP;
