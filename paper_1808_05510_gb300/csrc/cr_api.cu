@@ -759,12 +759,30 @@ cr_status build_lap(cr_problem* p, const cr_csr& c, DevLap& L) {
   return build_push(p, rows, diag, L, p->push[&L == &p->Lx ? 1 : 0]);
 }
 
-// Grid-wide form of the multigrid PCG (cr_mg_grid.cu) on the hierarchy H.  It
-// takes every SM in a cooperative launch, so it serves the problems that have
-// the GPU to themselves: one that caps its persistent Galerkin kernel
-// (galerkin_ctas, as the members of a sweep do) or asks for a cluster size
-// keeps the cluster kernel, of which many run side by side.  Leaves d.nb = 0
-// where it does not apply.
+// Grid-wide form of the multigrid PCG (cr_mg_grid.cu) on the hierarchy H.  A
+// problem that caps its persistent Galerkin kernel (galerkin_ctas, as the
+// members of a sweep do) or asks for a cluster size keeps the cluster kernel.
+// Leaves d.nb = 0 where it does not apply.
+//
+// A program may solve problems of its own side by side, on several streams, so
+// the CTAs leave room for those of other solves: their registers let two or
+// three share an SM, up to kMgGridHalf rows a solve takes half as many CTAs as
+// there are SMs, and tables that would keep a second CTA off the SM go to device
+// memory.  Measured on GB300, ms per solve on the u side for one handle and for
+// eight on eight threads (the 16-SM cluster kernel in brackets), against all SMs
+// with one CTA each:
+//   4,000 rows    float64  1.25, 0.27 [1.87, 0.27]; all SMs 1.28, 1.19
+//   7,500 rows    float64  1.36, 0.33 [1.97, 0.32]; all SMs 1.32, 1.22
+//   15,000 rows   float64  2.18, 0.59 [4.00, 0.63]; all SMs 2.08, 1.95
+//   25,000 rows   float64  2.16, 0.87 [5.45, 0.94]; all SMs 2.16, 2.03
+//   33,000 rows   mixed    3.78, 1.78 [7.74, 1.62]; all SMs 3.58, 3.27
+//   45,000 rows   mixed    3.43, 1.78 [8.16, 1.78]; all SMs 2.95, 2.66
+// 48 rows or more per CTA: with 16 a 400-row solve takes 0.97 instead of 0.88 ms, and
+// with 96 a 2,000-row one 1.17 instead of 1.12.
+constexpr int kMgGridHalf = 16000;   // (25,000 rows on half the CTAs: 2.56 ms instead of 2.16)
+// Rows per CTA up to which it has 256 threads, beyond 512: 33,000 rows on 152 CTAs, v side, 4.6
+// against 5.0 ms, 45,000 rows 18.5 against 16.4.
+constexpr int kMgGridFewRows = 236;
 cr_status build_mg_grid(cr_problem* p, const DevLap& L, const cr_mg::Hierarchy& H, const DevMg& h, DevMgGrid& out) {
   out = DevMgGrid{};
   if (p->opt.galerkin_ctas > 0 || p->opt.cluster_size > 0) return CR_OK;
@@ -775,9 +793,9 @@ cr_status build_mg_grid(cr_problem* p, const DevLap& L, const cr_mg::Hierarchy& 
   if (!coop || sms < 1) return CR_OK;
   const int n = h.lev[0].n, nlev = h.nlev, nc = h.nc, m = p->m;
   DevMgGrid d{};
-  d.nb = std::min(sms, std::max(1, (n + kMgGridRows - 1) / kMgGridRows));
+  d.nb = std::min(n <= kMgGridHalf ? std::max(1, sms / 2) : sms, std::max(1, (n + kMgGridRows - 1) / kMgGridRows));
   for (int l = 0; l < nlev; ++l) d.lev[l].chunk = (h.lev[l].n + d.nb - 1) / d.nb;
-  d.threads = kMgGridThreads;
+  d.threads = d.lev[0].chunk <= kMgGridFewRows ? kMgGridFew : kMgGridMany;
   // lanes per row: eight entries of a row are in flight per lane, so that most rows take one trip to L2
   auto lanes = [&](const std::vector<int>& rp, int rows, int threads) {
     int64_t mx = 0;
@@ -861,7 +879,7 @@ cr_status build_mg_grid(cr_problem* p, const DevLap& L, const cr_mg::Hierarchy& 
     TRY(dalloc(p, &W.dinv, (size_t)h.lev[l].n));
   }
   d.tab_bytes = (int)sm;
-  d.tab_smem = (int64_t)d.o_tab + sm <= kMgGridSmemMax ? 1 : 0;
+  d.tab_smem = (int64_t)d.o_tab + sm <= kMgGridSmemPair ? 1 : 0;
   d.smem = (size_t)d.o_tab + (d.tab_smem ? (size_t)sm : 0);
   if (d.smem > (size_t)kMgGridSmemMax) return CR_OK;
   if (!mg_grid_prepare(d)) return CR_OK;

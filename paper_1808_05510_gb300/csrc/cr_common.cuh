@@ -209,9 +209,11 @@ cudaError_t mg_pcg_launch(const PcgArgs& a, const DevMg& g, int side, cudaStream
 // the row split, the smoothed transfer S_l = P - w D^-1 (L + sigma M) P (rows
 // of level l, columns of level l+1) by its three parts on one pattern, its
 // transpose, and where the level's vectors and tables lie.
-constexpr int kMgGridThreads = 512;
-constexpr int kMgGridRows = 16;               // fewest level-0 rows per CTA
+constexpr int kMgGridFew = 256, kMgGridMany = 512;  // threads per CTA, by rows per CTA (see build_mg_grid)
+constexpr int kMgGridFewCtas = 3;             // CTAs per SM that the first form's registers leave room for
+constexpr int kMgGridRows = 48;               // fewest level-0 rows per CTA
 constexpr int kMgGridSmemMax = 224 * 1024;    // dynamic shared memory (about 1 KB is static)
+constexpr int kMgGridSmemPair = 112 * 1024;   // the same with two CTAs on an SM
 constexpr int kMgGridOwn0 = 16, kMgGridOwn = 7;  // own vectors of level 0 and of the levels below
 struct DevMgGridLevel {
   int chunk = 0;  // rows per CTA

@@ -1,7 +1,7 @@
 // Grid-wide multigrid-preconditioned CG for the ALS sub-problems (Sec. 2.3,
 // Eqs. ALS_linsys and ALS_linsys_v): the preconditioner of cr_mg.cu
 // (M^-1 = (1 / lam) V(V(.)), V one V-cycle of L + sigma I with two damped-Jacobi
-// sweeps before and after the coarse correction), spread over all SMs in one
+// sweeps before and after the coarse correction), spread over many SMs in one
 // cooperative launch.
 //
 // What bounds it.  A V-cycle is a chain of short dependent sweeps, so the time
@@ -16,18 +16,24 @@
 //    launch (own rows x nc, dense), which leaves no coarse-solve phase.  A
 //    three-level PCG iteration takes 19 barriers (the cluster kernel: 28), two more
 //    with the v side's Woodbury step.
-//  - All SMs.  The float64 pipe of GB300 issues one warp operation per 16 cycles,
+//  - Many SMs.  The float64 pipe of GB300 issues one warp operation per 16 cycles,
 //    so a level-0 sweep over 470 rows per CTA (16-CTA cluster, 7,530 voxels) is
-//    1.2 us of float64 arithmetic alone; 152 CTAs hold 50 rows each, and every
-//    table of the solve fits shared memory up to about 60,000 rows.
+//    1.2 us of float64 arithmetic alone; 76 CTAs hold 99 rows each, and every
+//    table of the solve fits shared memory up to about 30,000 rows.  The chain
+//    leaves an SM idle most of the time, so its registers and shared memory are
+//    kept to a half or a third of it, and CTAs of other handles' solves run beside
+//    it (the split and its figures: build_mg_grid in cr_api.cu).
 // Vectors that other CTAs gather live in global memory (L2) and are read with
 // ld.global.cg after a barrier; everything a row needs for itself stays in the
 // CTA's shared memory.  Barriers are those of cr_grid_bar.cuh (bounded).  Sums run
 // in a fixed order and every CTA forms the same scalars, so results repeat bit for
 // bit and all CTAs take the same branches.
 // Measured against the cluster kernel (ms per solve): 7,500 voxels, float64, v side
-// with 28 injections 2.92 -> 1.91; 45,000 voxels, float32, u side 6.42 -> 2.26.  An
-// iteration of that v side is 102 -> 50 us: 21 barriers of 1.2 us and 25 us between them.
+// with 28 injections 3.00 -> 2.08; 45,000 voxels, float32, u side 6.41 -> 2.62.  An
+// iteration of that v side is 102 -> 55 us: 21 barriers and the gathers between them.
+// With all 152 SMs for one solve these were 1.91 and 2.27 ms, and eight handles on
+// eight threads took turns: 1.22 ms a u-side solve of 7,500 voxels against 0.32 in
+// clusters, 0.33 now.
 #include <algorithm>
 
 #include "cr_common.cuh"
@@ -56,8 +62,8 @@ struct Int {
   static constexpr int value = N;
 };
 
-template <int KIND, class T>
-__global__ void __launch_bounds__(kMgGridThreads, 1) pcg_mg_grid_kernel(const PcgArgs A, const DevMg G, const DevMgGrid D) {
+template <int KIND, class T, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == kMgGridFew ? kMgGridFewCtas : 2) pcg_mg_grid_kernel(const PcgArgs A, const DevMg G, const DevMgGrid D) {
   const int b = blockIdx.x, nb = D.nb;
   const int tid = threadIdx.x, nth = blockDim.x;
   const int lane = tid & 31, wid = tid >> 5, nw = nth >> 5;
@@ -724,9 +730,15 @@ __global__ void __launch_bounds__(kMgGridThreads, 1) pcg_mg_grid_kernel(const Pc
   }
 }
 
-const void* mg_grid_fn(int side, bool f32) {
-  if (f32) return side == 0 ? (const void*)pcg_mg_grid_kernel<0, float> : (const void*)pcg_mg_grid_kernel<1, float>;
-  return side == 0 ? (const void*)pcg_mg_grid_kernel<0, double> : (const void*)pcg_mg_grid_kernel<1, double>;
+template <int THREADS>
+const void* mg_grid_fn_t(int side, bool f32) {
+  if (f32)
+    return side == 0 ? (const void*)pcg_mg_grid_kernel<0, float, THREADS> : (const void*)pcg_mg_grid_kernel<1, float, THREADS>;
+  return side == 0 ? (const void*)pcg_mg_grid_kernel<0, double, THREADS> : (const void*)pcg_mg_grid_kernel<1, double, THREADS>;
+}
+
+const void* mg_grid_fn(int side, bool f32, int threads) {
+  return threads == kMgGridFew ? mg_grid_fn_t<kMgGridFew>(side, f32) : mg_grid_fn_t<kMgGridMany>(side, f32);
 }
 
 }  // namespace
@@ -735,9 +747,9 @@ bool mg_grid_prepare(const DevMgGrid& D) {
   for (int side = 0; side < 2; ++side)
     for (int f = 0; f < 2; ++f) {
       int per = 0;
-      if (cudaFuncSetAttribute(mg_grid_fn(side, f == 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
+      if (cudaFuncSetAttribute(mg_grid_fn(side, f == 0, D.threads), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                kMgGridSmemMax) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, mg_grid_fn(side, f == 0), D.threads, D.smem) !=
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, mg_grid_fn(side, f == 0, D.threads), D.threads, D.smem) !=
               cudaSuccess ||
           per < 1) {
         cudaGetLastError();
@@ -755,7 +767,7 @@ cudaError_t mg_grid_launch(const PcgArgs& a, const DevMg& g, const DevMgGrid& d,
   DevMgGrid d2 = d;
   void* args[] = {&a2, &g2, &d2};
   count_launch();
-  return cudaLaunchCooperativeKernel(mg_grid_fn(side, a.fp32 != 0), dim3(d.nb), dim3(d.threads), args, d.smem, st);
+  return cudaLaunchCooperativeKernel(mg_grid_fn(side, a.fp32 != 0, d.threads), dim3(d.nb), dim3(d.threads), args, d.smem, st);
 }
 
 }  // namespace cr
