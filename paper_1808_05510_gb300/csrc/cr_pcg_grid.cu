@@ -46,9 +46,13 @@ namespace cr {
 
 namespace {
 
-// One CTA of 1,024 threads per SM with the 16-bit table, at most two of 512 with the general one:
-// (every further CTA lengthens the barriers and the sums behind them).
+// One CTA of 1,024 threads per SM with the 16-bit table; with the general one CTAs of 512, one per SM
+// or, from kGTwoRows rows on, two (up to six neighbours; more take 128 registers a thread).  A second
+// CTA lengthens the barriers and the sums behind them, and keeps twice the loads in flight: weighted
+// grids, us per iteration in float64 with one and with two, 60,000 rows 22 and 27, 500,000 60 and 59,
+// 3.0M 466 and 300.
 constexpr int kGThreads16 = 1024, kGThreads = 512;
+constexpr int kGTwoRows = 500000;
 constexpr int kMaxInj = 4096;  // injections of a problem
 
 struct GridPcg {
@@ -319,7 +323,7 @@ __device__ __forceinline__ T data_row(const GridPcg& a, const T* om, const doubl
 }
 
 template <class T, int KM, bool F16>
-__global__ void __launch_bounds__(F16 ? kGThreads16 : kGThreads, 1) pcg_grid_kernel(const GridPcg a) {
+__global__ void __launch_bounds__(F16 ? kGThreads16 : kGThreads, !F16 && KM == 6 ? 2 : 1) pcg_grid_kernel(const GridPcg a) {
   extern __shared__ double ys[];  // v side: y = s o (X^T v), m entries
   __shared__ double red[kParts], sums[3 * (F16 ? kGThreads16 : kGThreads)];
   T* xs = (T*)a.xs;
@@ -505,8 +509,8 @@ done:
 namespace cr {
 
 // Threads per block and largest block count that is co-resident for the kernel
-// variant (float32 or float64; neighbour table), at most one block of 1,024 or two
-// of 512 threads per SM (cooperative launch); 0 if it cannot run.
+// variant (float32 or float64; neighbour table), at most one block of 1,024 or one
+// or two of 512 threads per SM (cooperative launch); 0 if it cannot run.
 static int grid_threads(const DevLap& L) { return L.nbr16 ? kGThreads16 : kGThreads; }
 const void* grid_kernel_fn(bool fp32, const DevLap& L) {
   if (L.nbr16) return fp32 ? (const void*)pcg_grid_kernel<float, 6, true> : (const void*)pcg_grid_kernel<double, 6, true>;
@@ -528,7 +532,7 @@ int pcg_grid_blocks(bool fp32, int m, const DevLap& L) {
     cudaGetLastError();
     return 0;
   }
-  return sms * std::min(per, L.nbr16 ? 1 : 2);
+  return sms * std::min(per, L.nbr16 || L.n < kGTwoRows ? 1 : 2);
 }
 
 // vectors start at multiples of 16 rows, so that four rows load at once
