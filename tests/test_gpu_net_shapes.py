@@ -46,6 +46,20 @@ def test_bf16_gradients(env, dims, B):  # noqa: F811
     close(g, dWs, dbs, 1e-2)
 
 
+@pytest.mark.parametrize("dims", [(7, 9, 1), (70, 2, 1), (11, 1, 1), (67, 1, 1), (1, 6, 1), (1, 1, 5), (1, 1, 1), (4, 1, 6), (5, 9, 2),
+                                  (9, 5, 2), (3, 8, 7), (2, 7, 7), (6, 6, 7)])
+def test_thin_boxes(env, dims):  # noqa: F811
+    """Boxes of one- and two-dimensional grids, whose last extents are 1, and others walked along another axis."""
+    torch, cr = env
+    flat, x, t, mask = random_case(cr, sum(dims) + 1, dims, 3)
+    mask[0, 0, 0] = 1
+    out, loss, g = cr.ConvNet.check_f64(dims, flat, x, t, mask)
+    Ws, bs = unpack(flat)
+    ref, loss_ref, dWs, dbs = oracle_all(x, Ws, bs, t, mask)
+    assert np.linalg.norm(out - ref) <= 1e-10 * np.linalg.norm(ref)
+    close(g, dWs, dbs, 1e-10)
+
+
 def test_infinite_input_behind_dead_units(env):  # noqa: F811
     """Every unit that sees the infinite input is dead: its gradient is zero and the input adds
     nothing, as a large finite one does."""
