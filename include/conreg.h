@@ -58,8 +58,9 @@ typedef enum { CR_FP64 = 0, CR_MIXED = 1 } cr_precision;
  * with at most 32 injections the data term is added exactly by
  * Sherman-Morrison-Woodbury.  It runs on many SMs and leaves room on them for
  * solves of other problems on other streams, or in one thread-block cluster
- * when cluster_size or galerkin_ctas is set (as for members of a sweep); grids beyond one cluster's rows fall back to Jacobi.  CR_PRECOND_AUTO: multigrid in the float64
- * form; in the mixed form multigrid above 20,000 rows or for lambda >= 1e3
+ * when cluster_size or galerkin_ctas is set (as for members of a sweep); grids
+ * beyond one cluster's rows fall back to Jacobi.  CR_PRECOND_AUTO: multigrid in
+ * the float64 form; in the mixed form multigrid above 20,000 rows or for lambda >= 1e3
  * (where the Laplacian term dominates and Jacobi's iteration count grows),
  * Jacobi otherwise (there its many cheap float32 iterations are faster). */
 typedef enum {

@@ -1331,10 +1331,10 @@ PcgArgs pcg_args(cr_problem* p, int side, const double* b, double* x, int maxit,
 }
 
 // Kernel choice: the register-resident cluster kernel (float64) or the pushing
-// one (float32) while it applies (the whole solve on chip); beyond it the grid-wide kernel, which measured as fast
-// as the generic cluster kernel at 45k voxels and twice as fast at 127k
-// (16 SMs against all of them); pcg_kernel = 1 / 2 force the generic cluster
-// or the grid-wide kernel.
+// one (float32) while it applies (the whole solve on chip); beyond it the
+// grid-wide kernel, which runs on all SMs where the generic cluster kernel has 16
+// (127,000 voxels: twice as fast before its last changes, which halved its time);
+// pcg_kernel = 1 / 2 force the generic cluster or the grid-wide kernel.
 bool use_grid_pcg(const cr_problem* p, int side, bool fp32) {
   const DevLap& L = side == 0 ? p->Ly : p->Lx;
   if (p->opt.pcg_kernel == 2 || L.csize == 0) return true;
@@ -1342,14 +1342,20 @@ bool use_grid_pcg(const cr_problem* p, int side, bool fp32) {
   return fp32 ? p->push[side].csize == 0 : pcg_reg_vpt(L) == 0;
 }
 
-// One Jacobi-PCG solve on the cluster-resident kernel, or on the grid-wide
-// kernel (use_grid_pcg; that path waits for the result, to turn a grid
-// barrier timeout into CR_ETIMEOUT).
 // The automatic choice in float32: multigrid above this many rows, or from this
-// lambda on (measured on GB300 in the mixed form: at lambda = 100 on 7,530 voxels
-// Jacobi reaches relres 1e-6 in 11.5 s against multigrid's 15.0 s on the v side;
-// in the lambda sweep over 1 .. 1e6 on 15,000 voxels multigrid is faster overall
-// and leaves fewer members at the iteration cap).
+// lambda on.  The line was drawn on whole runs in the mixed form, with the cluster
+// kernels for both: at lambda = 100 on 7,530 voxels Jacobi reached relres 1e-6 in
+// 11.5 s against multigrid's 15.0 s on the v side; in the lambda sweep over
+// 1 .. 1e6 on 15,000 voxels multigrid was faster overall and left fewer members
+// at the iteration cap.  With the present kernels, one mixed solve from a zero
+// start, ms with Jacobi and with multigrid (us per iteration 2.7 to 5.5 and 57 to
+// 100 on both sides):
+//   7,500 rows, 28 injections, lambda 100: u 1.9, 1.5, v 6.4, 2.4; 1e3: u 4.9, 1.9, v 8.4, 2.7
+//   10,800 rows, 100 injections, lambda 100: u 1.2, 1.4, v 6.1, 8.9; 1e3: u 3.0, 1.9, v 9.4, 5.0
+//   23,900 rows, 28 injections, lambda 100: u 4.7, 2.5, v 20, 4.1; 1e3: u 11, 3.2, v 23, 4.5
+// So from a zero start multigrid would also pay below the line with few
+// injections; the line has not been drawn anew on whole runs, whose solves start
+// warm and take fewer iterations.
 constexpr int kMgAutoRows = 20000;
 constexpr double kMgAutoLambda = 1e3;
 
@@ -1358,13 +1364,14 @@ bool use_mg(const cr_problem* p, int side, bool fp32) {
   if (!(g.nlev >= 2 && (p->mgg[side].nb > 0 || g.smem[fp32 ? 0 : 1] > 0))) return false;
   if (p->opt.precond == CR_PRECOND_MULTIGRID) return true;
   if (p->opt.precond != CR_PRECOND_AUTO) return false;
-  // measured on GB300 (7,530 voxels): a multigrid iteration costs ~80-125 us (float32) / ~90-165 us
-  // (float64) against ~4-6 / ~9-13 us for Jacobi, while it cuts the iterations 10-50x; in float64
-  // that always pays, in float32 only where Jacobi's iteration count is large
+  // multigrid cuts the iterations 10-50x; at 45-80 us each (7,500 voxels) against 2.7-3.5 us for Jacobi
+  // in float32 and 9-13 us in float64, that always pays in float64 and in float32 where Jacobi takes many
   const DevLap& L = side == 0 ? p->Ly : p->Lx;
   return !fp32 || L.n > kMgAutoRows || p->lam >= kMgAutoLambda;
 }
 
+// One PCG solve on the kernel chosen above (the grid-wide Jacobi path waits for the
+// result, to turn a barrier timeout into CR_ETIMEOUT).
 cr_status run_pcg(cr_problem* p, int side, const double* b, double* x, int maxit, double tol, bool fp32) {
   const int kph = side == 0 ? CR_PHASE_PCG_KERNEL : CR_PHASE_PCG_KERNEL_V;
   if (use_mg(p, side, fp32)) {
@@ -1431,11 +1438,11 @@ cr_status launch_pcg_jacobi(cr_problem* p, int side, const double* b, double* x,
 // Mixed form of the sub-solves: float64 iterative refinement around the
 // float32 cluster PCG.  Each outer step forms the float64 residual
 // r = b - A_hat x, stops once |r| <= pcg_tol |b|, and otherwise solves
-// A_hat d = r from d = 0 in float32 (inner products in double-float) to
-// max(kMixedInnerTol, pcg_tol |b| / (2 |r|)) relative, then x += d.  An outer step that does not cut |r|
-// by 4x (float32 cannot resolve the system, e.g. at very large lambda) or the
-// step cap hands the solve over to the float64 kernel from the current x, so
-// the result meets the float64 tolerance either way.
+// A_hat d = r from d = 0 in float32 (inner products in double-float or float64) to
+// max(kMixedInnerTol, pcg_tol |b| / (4 |r|)) relative, then x += d.  An outer step
+// that does not cut |r| by 4x (float32 cannot resolve the system, e.g. at very
+// large lambda) or the step cap hands the solve over to the float64 kernel from
+// the current x, so the result meets the float64 tolerance either way.
 cr_status launch_pcg_mixed(cr_problem* p, int side, const double* b, double* x, int maxit) {
   cudaStream_t st = p->st;
   const DevLap& L = side == 0 ? p->Ly : p->Lx;
@@ -3112,7 +3119,7 @@ cr_status cr_svd_factors(cr_problem* p, double* Uh, int64_t ldu, double* sigma, 
 }
 
 // The solution pass runs on the tensor cores from this combined rank on, or from this many entries
-// (900^2: rank 16 0.13 against 0.11 ms, 24 0.135 against 0.137; 7,530^2: 1.6 against 2.6 ms at rank 1).
+// (ms, float64 pass and digits: 900^2 rank 24 0.133, 0.138, rank 40 0.170, 0.151; 7,569^2 rank 1 2.6, 1.6).
 constexpr int kPostTcRank = 24;
 constexpr int64_t kPostTcEntries = 1 << 22;
 

@@ -9,8 +9,8 @@
 // orthonormalisation in one cluster: eight launches for both grids and one read-back
 // (how many columns were accepted).  The float64 rate bounds the projections
 // (GB300: two FMAs per SM and clock): 12 n k FMAs per grid and step for a basis of
-// k columns, whatever the blocking; the blocking saves launches, round trips and
-// memory passes.  Factors of rank 240 on grids of 7,500 voxels, 28 injections, set and
+// k columns, and 3 n k for the coefficients behind them, whatever the blocking; the
+// blocking saves launches, round trips and memory passes.  Factors of rank 240 on grids of 7,500 voxels, 28 injections, set and
 // projected: 302 ms a pass, 100 of them in these products, before, and 177 ms after.
 #include <cooperative_groups.h>
 

@@ -59,26 +59,4 @@ __device__ __forceinline__ DF warp_sum_df(DF v) {
   return v;
 }
 
-// Sum NV per-thread DF values over the CTA; thread 0 stores them in out[].
-template <int NV>
-__device__ __forceinline__ void block_sum_df(DF (&v)[NV], DF* scr, DF* out) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int q = 0; q < NV; ++q) v[q] = warp_sum_df(v[q]);
-  if (lane == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) scr[wid * NV + q] = v[q];
-  }
-  __syncthreads();
-  if (wid == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      DF t = lane < nw ? scr[lane * NV + q] : DF{0.f, 0.f};
-      t = warp_sum_df(t);
-      if (lane == 0) out[q] = t;
-    }
-  }
-}
-
-
 }  // namespace cr

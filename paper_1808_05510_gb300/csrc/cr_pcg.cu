@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(kPcgThreads, 1) pcg_reg_kernel(const PcgArgs A
   const double lam = A.lam;
   const double c = A.coef[0];
   const double d = A.coef[1];
-  const double e = (d - c * c);
+  const double e = d - c * c;
   if (threadIdx.x == 0) {
     zero[0] = 0;
     zero[1] = 0;
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kPcgThreads, 1) pcg_reg_kernel(const PcgArgs A
           }
         }
       }
-      dpc[k] = (L.diag[i] + c);
+      dpc[k] = L.diag[i] + c;
       double dd = A.lam * (L.l2diag[i] + 2.0 * c * L.diag[i] + d);
       if (KIND == 0) {
         double o = 0.0;
@@ -402,38 +402,38 @@ __global__ void __launch_bounds__(kPcgThreads, 1) pcg_reg_kernel(const PcgArgs A
     }
     return ((v[0] + v[1]) + (v[2] + v[3])) + (v[4] + v[5]);
   };
-  // v side: partial X^double of the buffer in shared memory
+  // v side: partial X^T of the buffer in shared memory
   auto ypartial = [&](double* buf) {
     if (KIND == 1) {
       const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
       for (int a = wid; a < m; a += nw) {
         const int p0 = A.X.lx_ptr[rank * m + a], p1 = A.X.lx_ptr[rank * m + a + 1];
-          double acc = 0.0;
-          for (int q = p0 + lane; q < p1; q += 32) acc += A.X.lx_val[q] * (double)buf[A.X.lx_row[q]];
-          acc = warp_sum(acc);
-          if (lane == 0) ypart[a] = acc;
+        double acc = 0.0;
+        for (int q = p0 + lane; q < p1; q += 32) acc += A.X.lx_val[q] * buf[A.X.lx_row[q]];
+        acc = warp_sum(acc);
+        if (lane == 0) ypart[a] = acc;
       }
     }
   };
   auto gather = [&]() {
     if (KIND == 1) {
       for (int a = threadIdx.x; a < m; a += blockDim.x) {
-          double pv[kMaxCluster];
+        double pv[kMaxCluster];
 #pragma unroll
-          for (int rr = 0; rr < kMaxCluster; ++rr) pv[rr] = rr < C ? cl.map_shared_rank(ypart, (unsigned)rr)[a] : 0.0;
-          double t = 0.0;
+        for (int rr = 0; rr < kMaxCluster; ++rr) pv[rr] = rr < C ? cl.map_shared_rank(ypart, (unsigned)rr)[a] : 0.0;
+        double t = 0.0;
 #pragma unroll
-          for (int rr = 0; rr < kMaxCluster; ++rr) t += pv[rr];
-          sY[a] = sS[a] * t;
+        for (int rr = 0; rr < kMaxCluster; ++rr) t += pv[rr];
+        sY[a] = sS[a] * t;
       }
       __syncthreads();
     }
   };
   auto data = [&](int k, double ui) -> double {
     if (KIND == 0) return omt[k] * ui;
-      double acc = 0.0;
-      for (int q = xr0[k]; q < xr1[k]; ++q) acc += A.X.xr_val[q] * sY[A.X.xr_col[q]];
-      return acc;
+    double acc = 0.0;
+    for (int q = xr0[k]; q < xr1[k]; ++q) acc += A.X.xr_val[q] * sY[A.X.xr_col[q]];
+    return acc;
   };
 
   // r0 = b - A x0

@@ -22,8 +22,9 @@
 // Every block adds the per-block partial sums itself, in one fixed order, so
 // all blocks hold bit-identical scalars and take identical decisions.
 // T = float: float32 vectors and arithmetic with double-float (two-float)
-// accumulation of the inner products per thread, float64 between threads; T = double: float64 throughout (on
-// GB300 the float64 form is bound by float64 arithmetic, not by HBM).
+// accumulation of the inner products per thread, float64 between threads;
+// T = double: float64 throughout (on GB300 the float64 form is bound by float64
+// arithmetic, not by HBM).
 // Neighbour tables: a unit-weight graph Laplacian with at most six neighbours
 // per row, none further than 32,767 rows away, stores the six distances as
 // 16-bit integers (12 B per row instead of 24 B, and L_ii is their count);

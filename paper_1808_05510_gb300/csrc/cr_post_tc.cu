@@ -22,13 +22,15 @@
 // makes E at most 0.57 of the float64 sum's bound.  Tiles of 64 x 64 entries in which
 // some T is smaller (rows whose large entries do not meet, and the sign and size of W
 // there) go to the float64 pass, the others come from the digits.
-// Measured (7,530^2 entries, ms per report): rank 100 against rank 140 25.2 -> 5.8 (0.4 of
-// them the check), before the check rank 100 alone 11.5 -> 2.3, rank 1 2.6 -> 1.5 (what the statistics' float64
-// operations take); W's error against extended precision 6.6e-16 -> 3.9e-16 at rank
-// 140.  A warp holds 16 x 16 entries (eight levels: 64 accumulators), eight warps a
+// Measured (7,530^2 entries, ms per report): rank 100 against rank 140 25.2 -> 5.8 (0.4
+// of them the check), rank 100 alone 11.8 -> 2.5, rank 1 2.6 -> 1.6 (what the
+// statistics' float64 operations take); W's error against extended precision
+// 6.6e-16 -> 3.9e-16 at rank 140.  A warp holds 16 x 16 entries (eight levels: 64 accumulators), eight warps a
 // CTA and two CTAs an SM; W and the statistics wait in shared memory meanwhile (kept
-// in registers they spilled: 5.8 ms; one CTA of 64 x 64 entries: 6.7 ms).  Bound now
-// by the issue of the matrix instructions and, a third, by the float64 epilogue.
+// in registers they spilled: 5.8 ms; one CTA of 64 x 64 entries: 6.7 ms).  At rank 100
+// alone the float64 pipe is 63 % busy (level sums, statistics) and the tensor pipe 41 %,
+// in turns: the two CTAs of an SM overlap the phases only in part.  The check's 0.21 ms
+// are latency of its operand loads.
 #include <cuda_bf16.h>
 
 #include <algorithm>

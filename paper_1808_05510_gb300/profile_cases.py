@@ -3,9 +3,10 @@
     python -m paper_1808_05510_gb300.profile_cases pcg fp64|mixed [jacobi|auto]
         one u-side and one v-side ALS solve (Eqs. ALS_linsys, ALS_linsys_v) for the
         first ALS vector v = R_0^T 1 / |R_0^T 1|, to relative residual 1e-8, twice;
-        jacobi (default): Jacobi PCG on both sides; auto: the automatic choice
-        (multigrid PCG on the v side, pcg_mg_kernel); prints iterations and the
-        CUDA-event time of each solve
+        jacobi (default): Jacobi PCG on both sides (pcg_reg_kernel, mixed
+        pcg_push_kernel); auto: the automatic choice (fp64: multigrid PCG on both
+        sides, pcg_mg_grid_kernel); prints iterations and the CUDA-event time of
+        each solve
     python -m paper_1808_05510_gb300.profile_cases galerkin fp64|mixed [eigen|jacobi]
         two Galerkin projections (Eq. Proj_Sylv) at rank 60 from a float64 greedy run,
         in the eigenbasis form (default) or the original-basis Jacobi form
@@ -15,9 +16,9 @@
     python -m paper_1808_05510_gb300.profile_cases assembly tc
         three tensor-core assemblies of G_a = U^T diag(Omega_a) U at rank 100
     python -m paper_1808_05510_gb300.profile_cases post fp64
-        three solution passes (W = U Z V^T in float64 tiles, projected onto W >= 0,
-        statistics only) at rank 100 with random orthonormal U, V; prints the
-        CUDA-event time of each call
+        three solution passes (W = U Z V^T from digits, post_check_kernel and
+        post_tc_kernel, projected onto W >= 0, statistics only) at rank 100 with
+        random orthonormal U, V; prints the CUDA-event time of each call
     python -m paper_1808_05510_gb300.profile_cases pcg_stress fp32|fp64 [solves]
         u-side ALS solves on the ~4M-voxel stress shell (grid-wide PCG, vectors in
         HBM): fp32 = one float32 grid solve to 1e-5 inside the mixed form's
