@@ -566,7 +566,7 @@ def measure_post(p, args, prec, reps: int = 5):
             "entries_per_s": entries / (rep_ms / 1e3), "negative_entries": rep["n_negative"],
             "negative_mass_rms": (rep["neg_fro2"] / entries) ** 0.5,
             "roofline": {"bound": "alu", "achieved": achieved, "peak": FP64_TFLOPS, "unit": "TFLOP/s",
-                         "frac": achieved / FP64_TFLOPS, "kernel": "post_tile_kernel (float64 W = U Z V^T tiles)",
+                         "frac": achieved / FP64_TFLOPS, "kernel": "post_tc_kernel (W = U Z V^T from digits on the tensor cores, float64 accuracy)",
                          "peak_kind": "of derived (152 SMs x 2 FP64 FMA/clk x 2.07 GHz)",
                          "flops_per_call": flops}}
 
