@@ -565,7 +565,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == kMgGridFew ? kMgGridFewCta
     // The operator is then applied to the u that enters x.  Its data term also follows from y
     // (S X^T u = Q y), and t from stored rows of (L + cI) MX Q, which would save a phase, but in the
     // span of X u0 is much larger than u, and A u then differs from that of the rounded u by u0's
-    // rounding: solves for 1e-13 stopped at 1e-12 of the right side, float32 ones for 1e-5 at 1e-4.
+    // rounding: float64 solves for 1e-13 (3,000 rows, 5 to 32 injections, lambda 1 to 300) left
+    // 1.4e-13 to 4.7e-12 of the right side, against 5e-14 to 1.2e-13.
     for (int idx = tid; idx < n0 * m; idx += nth) {
       const int li = idx / m, q = idx % m, i = beg0 + li;
       const T* row = mx + (size_t)i * m;
