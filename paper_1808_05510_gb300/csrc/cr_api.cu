@@ -1905,9 +1905,9 @@ cr_status do_project(cr_problem* p, double tol, cr_proj_info* info) {
         }
         CUCHK(p, cudaMemsetAsync(p->gbar, 0, 2 * sizeof(unsigned), st));
         CUCHK(p, cudaMemsetAsync(p->gerr, 0, sizeof(int), st));
-        // the whole system to the tolerance itself (a tighter first target costs more
-        // iterations than the refinements it saves); a correction to half of it
-        const double t2 = (ref == 0 ? 1.0 : 0.25) * tol * tol * fn2;
+        // to half the tolerance: what a refinement left while the bases' rounding made one
+        // necessary as a rule; with bases accurate to 1e-15 the first CG is the only one
+        const double t2 = 0.25 * tol * tol * fn2;
         CUCHK(p, galerkin_cg_launch(p->gal_nb, j, p->m, ld, p->lam, p->A1, p->eA2t, p->B1, p->eB2t, p->G, p->eHt,
                                     p->eFt, p->eDen, p->eZt, p->gR, p->gP, p->gT, p->gQ, p->gZB2, p->gZB1, p->gZH,
                                     p->gGw, p->gzb, p->gpart, p->gbar, p->gerr, t2, std::max(1, maxit - k), p->gout,
