@@ -3118,10 +3118,13 @@ cr_status cr_svd_factors(cr_problem* p, double* Uh, int64_t ldu, double* sigma, 
   return sync(p);
 }
 
-// The solution pass runs on the tensor cores from this combined rank on, or from this many entries
-// (ms, float64 pass and digits: 900^2 rank 24 0.133, 0.138, rank 40 0.170, 0.151; 7,569^2 rank 1 2.6, 1.6).
-constexpr int kPostTcRank = 24;
-constexpr int64_t kPostTcEntries = 1 << 22;
+// The solution pass runs on the tensor cores from this many entries on, or from fewer with this many
+// entries times columns (those of W and of the reference): the digits, the check and the second pass
+// take five launches more.  Measured, ms in float64 and from digits:
+//   625^2 rank 32 0.087, 0.116, rank 64 0.131, 0.144, rank 140 0.230, 0.238
+//   900^2 rank 24 0.134, 0.141, rank 48 0.171, 0.152, ranks 16 and 16 0.211, 0.266, 24 and 24 0.280, 0.275
+//   1,600^2 rank 8 0.185, 0.193, rank 16 0.185, 0.168; 2,500^2 rank 8 0.353, 0.274
+constexpr int64_t kPostTcEntries = 1 << 22, kPostTcFewest = 600000, kPostTcWork = 36000000;
 
 cr_status cr_solution_report(cr_problem* p, int32_t nonneg, int32_t jr, const double* Ur, int64_t ldur,
                              const double* Zr, int64_t ldzr, const double* Vr, int64_t ldvr, double* W, int64_t ldw,
@@ -3174,7 +3177,9 @@ cr_status cr_solution_report(cr_problem* p, int32_t nonneg, int32_t jr, const do
   }
   // tensor-core form: digits of the four factors, and the float64 pass behind it for
   // the tiles that they do not hold
-  bool tc = j > 0 && (j + jr >= kPostTcRank || out->entries >= kPostTcEntries) && post_tc_blocks() > 0;
+  const bool large = out->entries >= kPostTcEntries ||
+                     (out->entries >= kPostTcFewest && out->entries * (j + jr) >= kPostTcWork);
+  bool tc = j > 0 && large && post_tc_blocks() > 0;
   auto dig_rows = [&](int k) { return k % 2 == 0 ? ny : nx; };  // P, V, Pr, Vr
   auto dig_rank = [&](int k) { return k < 2 ? j : jr; };
   if (tc) {

@@ -23,7 +23,7 @@ def cr():
 
 
 def passes(cr, prec, precond, kernel):
-    p = synth.masked3d()
+    p = synth.masked3d(box=14, n_target=1200)  # enough entries for the solution pass's digits
     rng = np.random.default_rng(1)
     u, v = synth.random_unit(p.ny, 3), synth.random_unit(p.nx, 4)
     out = []

@@ -50,7 +50,7 @@ def factors(kind, ny, nx, j):
 
 
 @pytest.mark.parametrize("kind", ["bumps0.1", "bumps0.08", "bumps0.05", "bumps0.02", "decay", "apart"])
-@pytest.mark.parametrize("sides,j", [((13, 15, 14, 11), 24), ((20, 16, 9, 15), 115)])
+@pytest.mark.parametrize("sides,j", [((13, 15, 14, 11), 24), ((20, 16, 9, 15), 115), ((27, 31, 25, 32), 60)])
 def test_entries_to_their_own_size(cr, kind, sides, j):
     p = synth.rect2d(shape_y=sides[:2], shape_x=sides[2:], m=3)
     U, Z, V = factors(kind, p.ny, p.nx, j)

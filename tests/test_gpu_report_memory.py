@@ -27,7 +27,7 @@ def cr():
 
 @pytest.mark.parametrize("jr", [0, 40])
 def test_report_without_room_for_digits(cr, monkeypatch, jr):
-    p = synth.masked3d()
+    p = synth.masked3d(box=14, n_target=1200)  # enough entries for the digits
     rng = np.random.default_rng(1)
     j = 30
     U, Z, V = rng.standard_normal((p.ny, j)), rng.standard_normal((j, j)), rng.standard_normal((p.nx, j))
